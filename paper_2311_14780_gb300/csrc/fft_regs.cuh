@@ -37,7 +37,46 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
 __device__ __forceinline__ float2 cconjmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.x, b.y, -a.y * b.x));
 }
-__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+// (rounded on its own: the compiler may not fuse it into a following addition, so that every pass
+// that scales and then adds rounds alike)
+__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(__fmul_rn(a.x, s), __fmul_rn(a.y, s)); }
+
+// Two complex numbers, one per lane of the packed FP32 instructions (fadd2 / fmul2 / ffma2 of
+// sm_100 and later): the same element of two independent fields.  Every operation below rounds each
+// lane exactly like its float2 counterpart above.
+struct __align__(16) cpair {
+  float2 re, im;
+};
+__device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ cpair cadd(cpair a, cpair b) { return {__fadd2_rn(a.re, b.re), __fadd2_rn(a.im, b.im)}; }
+__device__ __forceinline__ cpair csub(cpair a, cpair b) {
+  return {__fadd2_rn(a.re, neg2(b.re)), __fadd2_rn(a.im, neg2(b.im))};
+}
+// both lanes times one complex number
+__device__ __forceinline__ cpair cmul(cpair a, float2 b) {
+  const float2 bx = splat(b.x), by = splat(b.y);
+  return {__ffma2_rn(a.re, bx, neg2(__fmul2_rn(a.im, by))), __ffma2_rn(a.re, by, __fmul2_rn(a.im, bx))};
+}
+__device__ __forceinline__ cpair cmulc(cpair a, float2 b) {
+  const float2 bx = splat(b.x), by = splat(b.y);
+  return {__ffma2_rn(a.re, bx, __fmul2_rn(a.im, by)), __ffma2_rn(a.im, bx, neg2(__fmul2_rn(a.re, by)))};
+}
+// one complex number times both lanes, and its conjugate times both lanes
+__device__ __forceinline__ cpair cmul(float2 a, cpair b) {
+  const float2 ax = splat(a.x), ay = splat(a.y);
+  return {__ffma2_rn(ax, b.re, neg2(__fmul2_rn(ay, b.im))), __ffma2_rn(ax, b.im, __fmul2_rn(ay, b.re))};
+}
+__device__ __forceinline__ cpair cconjmul(float2 a, cpair b) {
+  const float2 ax = splat(a.x), ay = splat(a.y);
+  return {__ffma2_rn(ax, b.re, __fmul2_rn(ay, b.im)), __ffma2_rn(ax, b.im, neg2(__fmul2_rn(ay, b.re)))};
+}
+// lane by lane real factors; like the scalar form, rounded on its own (scalar multiplications: measured,
+// the compiler fuses a packed one into a following packed addition even when both are .rn)
+__device__ __forceinline__ cpair cscale(cpair a, float2 s) {
+  return {make_float2(__fmul_rn(a.re.x, s.x), __fmul_rn(a.re.y, s.y)),
+          make_float2(__fmul_rn(a.im.x, s.x), __fmul_rn(a.im.y, s.y))};
+}
 
 // cos(2*pi*i/32) for i in [0, 8]
 __host__ __device__ constexpr double kCos32(int i) {
@@ -88,18 +127,45 @@ __device__ __forceinline__ float2 twiddle_const(float2 x) {
   }
 }
 
+template <int N, bool INV, int K>
+__device__ __forceinline__ cpair twiddle_const(cpair x) {
+  constexpr int a = ((K * (32 / N)) % 32 + 32) % 32;
+  if constexpr (a == 0) {
+    return x;
+  } else if constexpr (a == 16) {
+    return {neg2(x.re), neg2(x.im)};
+  } else if constexpr (a == 8) {
+    return INV ? cpair{neg2(x.im), x.re} : cpair{x.im, neg2(x.re)};
+  } else if constexpr (a == 24) {
+    return INV ? cpair{x.im, neg2(x.re)} : cpair{neg2(x.im), x.re};
+  } else {
+    constexpr float c = (float)cos32(a);
+    constexpr float s = INV ? (float)sin32(a) : -(float)sin32(a);   // W = c + i*s
+    return {__ffma2_rn(x.re, splat(c), neg2(__fmul2_rn(x.im, splat(s)))),
+            __ffma2_rn(x.re, splat(s), __fmul2_rn(x.im, splat(c)))};
+  }
+}
+// x * (-i) (forward) or x * (+i) (INV)
+template <bool INV> __device__ __forceinline__ float2 quarter_turn(float2 x) {
+  return INV ? make_float2(-x.y, x.x) : make_float2(x.y, -x.x);
+}
+template <bool INV> __device__ __forceinline__ cpair quarter_turn(cpair x) {
+  return INV ? cpair{neg2(x.im), x.re} : cpair{x.im, neg2(x.re)};
+}
+
 // In-place DFT of N values a[0], a[S], ..., a[(N-1)S]; natural order in and out.
 template <int N, int S, bool INV>
 struct Dft {
-  static __device__ __forceinline__ void run(float2* a) {
-    float2 e[N / 2], o[N / 2];
+  template <class V>
+  static __device__ __forceinline__ void run(V* a) {
+    V e[N / 2], o[N / 2];
 #pragma unroll
     for (int k = 0; k < N / 2; ++k) { e[k] = a[(2 * k) * S]; o[k] = a[(2 * k + 1) * S]; }
     Dft<N / 2, 1, INV>::run(e);
     Dft<N / 2, 1, INV>::run(o);
     static_for<0, N / 2>([&](auto kc) {
       constexpr int k = decltype(kc)::value;
-      const float2 w = twiddle_const<N, INV, k>(o[k]);
+      const V w = twiddle_const<N, INV, k>(o[k]);
       a[k * S] = cadd(e[k], w);
       a[(k + N / 2) * S] = csub(e[k], w);
     });
@@ -107,12 +173,13 @@ struct Dft {
 };
 template <int S, bool INV>
 struct Dft<4, S, INV> {
-  static __device__ __forceinline__ void run(float2* a) {
-    const float2 x0 = a[0], x1 = a[S], x2 = a[2 * S], x3 = a[3 * S];
-    const float2 s02 = cadd(x0, x2), d02 = csub(x0, x2);
-    const float2 s13 = cadd(x1, x3), d13 = csub(x1, x3);
+  template <class V>
+  static __device__ __forceinline__ void run(V* a) {
+    const V x0 = a[0], x1 = a[S], x2 = a[2 * S], x3 = a[3 * S];
+    const V s02 = cadd(x0, x2), d02 = csub(x0, x2);
+    const V s13 = cadd(x1, x3), d13 = csub(x1, x3);
     // forward: X1 = d02 - i d13, X3 = d02 + i d13 ; inverse swaps the signs
-    const float2 jd13 = INV ? make_float2(-d13.y, d13.x) : make_float2(d13.y, -d13.x);
+    const V jd13 = quarter_turn<INV>(d13);
     a[0] = cadd(s02, s13);
     a[S] = cadd(d02, jd13);
     a[2 * S] = csub(s02, s13);
@@ -121,8 +188,9 @@ struct Dft<4, S, INV> {
 };
 template <int S, bool INV>
 struct Dft<2, S, INV> {
-  static __device__ __forceinline__ void run(float2* a) {
-    const float2 x0 = a[0], x1 = a[S];
+  template <class V>
+  static __device__ __forceinline__ void run(V* a) {
+    const V x0 = a[0], x1 = a[S];
     a[0] = cadd(x0, x1);
     a[S] = csub(x0, x1);
   }

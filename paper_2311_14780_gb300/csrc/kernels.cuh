@@ -1174,11 +1174,20 @@ __host__ __device__ constexpr int row_adj_l_smem(int M, int rpb, bool probe_l2 =
 // kRowAdjL2Threads threads) is compiled for two blocks per SM instead of one.
 constexpr int kRowAdjL2Threads = 160;
 
-// Next position of this split after b whose index is valid, or -1 (uniform over the block).
+// acc += conj(o) v, in the operations of the pair passes (pair.cuh).
+__device__ __forceinline__ void acc_conjmul(float2& acc, float2 o, float2 v) {
+  acc.x = fmaf(o.x, v.x, fmaf(o.y, v.y, acc.x));
+  acc.y = fmaf(o.x, v.y, fmaf(-o.y, v.x, acc.y));
+}
+
+// Positions are dealt to the splits in pairs (2p, 2p + 1), p = split, split + nsplit, ..., the order of
+// the pair passes.  Next position of this split after b whose index is valid, or -1 (uniform over the
+// block); before_split(split, nsplit) comes before the first.
+__device__ __forceinline__ int before_split(int split, int nsplit) { return 2 * (split - nsplit) + 1; }
 __device__ __forceinline__ int next_pos(const int2* spos, int b, int nb, int nsplit) {
-  for (int bb = b + nsplit; bb < nb; bb += nsplit)
-    if (spos[bb].x >= 0) return bb;
-  return -1;
+  do b = (b & 1) ? 2 * ((b >> 1) + nsplit) : b + 1;
+  while (b < nb && spos[b].x < 0);
+  return b < nb ? b : -1;
 }
 
 // Copies of the rpb object rows of position (y, x) (8-byte pieces: x may be odd).
@@ -1234,7 +1243,7 @@ __device__ __forceinline__ void row_adj_l_body(const float2* __restrict__ O, con
   float2 acc[N2];
 #pragma unroll
   for (int n2 = 0; n2 < N2; ++n2) acc[n2] = make_float2(0.f, 0.f);
-  int b = next_pos(spos, split - nsplit, a.nb, nsplit);
+  int b = next_pos(spos, before_split(split, nsplit), a.nb, nsplit);
   if (b >= 0) prefetch(b, 0);
   for (int buf = 0; b >= 0; buf ^= 1) {
     cp_async_wait<0>();
@@ -1252,11 +1261,10 @@ __device__ __forceinline__ void row_adj_l_body(const float2* __restrict__ O, con
 #pragma unroll
     for (int n2 = 0; n2 < N2; ++n2) {
       const int c = t + N1 * n2;
-      const float2 gp = cconjmul(orow[c], v[n2]);                       // conj(p) chi
-      acc[n2].x = fmaf(s, gp.x, acc[n2].x);
-      acc[n2].y = fmaf(s, gp.y, acc[n2].y);
+      const float2 sv = cscale(v[n2], s);                               // sigma chi
+      acc_conjmul(acc[n2], orow[c], sv);                                // conj(p) sigma chi
       const float2 pv = PL2 ? __ldg(Prow + c) : Psm[vec * F + c];
-      reg[c] = cscale(cconjmul(pv, v[n2]), s);                          // conj(sigma P) chi
+      reg[c] = cconjmul(pv, sv);                                        // conj(P) sigma chi
     }
     __syncthreads();
     float2* dst = S + (((long long)b * a.C + slot0) * F + row0) * F;      // the block's rpb rows, contiguous
@@ -1340,7 +1348,7 @@ __device__ __forceinline__ void row_adj_w_body(const float2* __restrict__ O, con
   float2 acc[16];
 #pragma unroll
   for (int n2 = 0; n2 < 16; ++n2) acc[n2] = make_float2(0.f, 0.f);
-  int b = next_pos(spos, split - nsplit, a.nb, nsplit);
+  int b = next_pos(spos, before_split(split, nsplit), a.nb, nsplit);
   if (b >= 0) prefetch(b, 0);
   for (int buf = 0; b >= 0; buf ^= 1) {
     cp_async_wait<0>();
@@ -1355,10 +1363,9 @@ __device__ __forceinline__ void row_adj_w_body(const float2* __restrict__ O, con
 #pragma unroll
     for (int n2 = 0; n2 < 16; ++n2) {
       const int c = t + 32 * n2;
-      const float2 gp = cconjmul(orow[c], v[n2]);                       // conj(p) chi
-      acc[n2].x = fmaf(s, gp.x, acc[n2].x);
-      acc[n2].y = fmaf(s, gp.y, acc[n2].y);
-      reg[c] = cscale(cconjmul(__ldg(Prow + c), v[n2]), s);             // conj(sigma P) chi
+      const float2 sv = cscale(v[n2], s);                               // sigma chi
+      acc_conjmul(acc[n2], orow[c], sv);                                // conj(p) sigma chi
+      reg[c] = cconjmul(__ldg(Prow + c), sv);                           // conj(P) sigma chi
     }
     __syncthreads();
     float2* dst = S + (((long long)b * a.C + slot0) * F + row0) * F;
@@ -1427,7 +1434,7 @@ k_row_fwd_l(const float2* __restrict__ O, const float2* __restrict__ P, float2* 
   }
   const float2* Ol = O + a.obj_off[l];
   const int Wl = a.obj_w[l];
-  int b = next_pos(spos, split - nsplit, a.nb, nsplit);
+  int b = next_pos(spos, before_split(split, nsplit), a.nb, nsplit);
   if (b >= 0) {
     prefetch_orows<F>(Ol, Wl, spos[b], row0, rpb, Ost);
     cp_async_commit();
@@ -1489,7 +1496,7 @@ k_row_fwd_w(const float2* __restrict__ O, const float2* __restrict__ P, float2* 
   const float2* Ol = O + a.obj_off[l];
   const int Wl = a.obj_w[l];
   const int oc = (t & 15) + 256 * (t >> 4);           // output column of x[0] (then + 16 j)
-  int b = next_pos(spos, split - nsplit, a.nb, nsplit);
+  int b = next_pos(spos, before_split(split, nsplit), a.nb, nsplit);
   if (b >= 0) {
     prefetch_orows<F>(Ol, Wl, spos[b], row0, rpb, Ost);
     cp_async_commit();
@@ -1524,7 +1531,7 @@ __global__ void k_sum_splits(const float2* __restrict__ part, int nsplit, long l
 // patches overlap the tile are listed first (ascending), then added four at a time with
 // their loads issued together.   grid (tiles of the largest box, L)
 // ---------------------------------------------------------------------------------------
-template <int F>
+template <int F, bool PAIR = false>
 __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, float2* __restrict__ gO, const KArgs& a,
                                                 const uint3 bid) {
   __shared__ int2 spos[kMaxB];
@@ -1570,12 +1577,14 @@ __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, fl
       const int b = i0 + pp < n ? list[i0 + pp] : -1;
       const int y = b >= 0 ? spos[b].x : 0, x = b >= 0 ? spos[b].y : 0;
       const bool in_x = b >= 0 && ox >= x && ox < x + F;
-      const float2* src = S + ((long long)(b >= 0 ? b : 0) * a.C + slot0) * F * F + (ox - x);
+      const int bs = b >= 0 ? b : 0;
+      const float2* src = PAIR ? S + ((long long)(bs >> 1) * a.C + slot0) * 2 * F * F + (bs & 1) * F + (ox - x)
+                               : S + ((long long)bs * a.C + slot0) * F * F + (ox - x);
 #pragma unroll
       for (int k = 0; k < kTile / 8; ++k) {
         const int oy = oy0 + ty0 + 8 * k;
         const bool ok = in_x && oy >= y && oy < y + F;
-        v[pp][k] = ok ? src[(long long)(oy - y) * F] : make_float2(0.f, 0.f);
+        v[pp][k] = ok ? src[(long long)(oy - y) * (PAIR ? 2 * F : F)] : make_float2(0.f, 0.f);
       }
     }
 #pragma unroll
@@ -1594,12 +1603,13 @@ __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, fl
   }
 }
 
-template <int F>
+// PAIR: the slots of the pair passes (rows of 2 F float2: lane 0's row, then lane 1's).
+template <int F, bool PAIR>
 __global__ void __launch_bounds__(256)
 k_obj_grad_l(const float2* __restrict__ S, float2* __restrict__ gO, KArgs a) {
   pdl_wait();
   pdl_trigger();
-  obj_grad_l_body<F>(S, gO, a, blockIdx);
+  obj_grad_l_body<F, PAIR>(S, gO, a, blockIdx);
 }
 
 // ---------------------------------------------------------------------------------------

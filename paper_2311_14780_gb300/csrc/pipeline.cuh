@@ -1,8 +1,10 @@
 // Orchestration of one compute call for a fixed frame size F: loops over position batches
 // and mode chunks and launches the kernels of kernels.cuh on the caller's stream.
 #pragma once
+#include <algorithm>
 #include <mutex>
 
+#include "pair.cuh"
 #include "plan.h"
 #include "resident.cuh"
 #include "serve_multi.cuh"
@@ -50,6 +52,26 @@ int launch_cols_s(ptycho_plan& p, bool fwd, bool store, cudaStream_t cs, float2*
   return PTYCHO_OK;
 }
 
+// Row adjoint of the pair passes: one warp per block with one mode, else the block of all modes in the
+// launch class of its size.
+template <int F>
+int launch_row_adj_pair(ptycho_plan& p, cudaStream_t cs, const CallArgs& c, float2* S, float2* gPs, const KArgs& a,
+                        int nsplit) {
+  float4* S4 = reinterpret_cast<float4*>(S);
+  if (p.M == 1) {
+    PTY_LAUNCH(p, kRowAdj, cs,
+               launch_pdl(k_row_adj_p1<F>, dim3(F / PairCfg<F>::VPW, p.L, nsplit), 32, row_adj_p1_smem<F>(), cs, c.O, c.P,
+                          S4, gPs, (long long)p.P_numel, a, nsplit));
+    return PTYCHO_OK;
+  }
+  const int ct = PairCfg<F>::T * p.M * p.rpb_pair, feeders = row_adj_p_feeders(ct);
+  auto* k = feeders == 1 ? k_row_adj_p<F, 1> : k_row_adj_p<F, 2>;
+  PTY_LAUNCH(p, kRowAdj, cs,
+             launch_pdl(k, dim3(F / p.rpb_pair, p.L, nsplit), ct + 32 * feeders, row_adj_p_smem<F>(p.M, p.rpb_pair), cs,
+                        c.O, c.P, S4, gPs, (long long)p.P_numel, a, p.rpb_pair, nsplit));
+  return PTYCHO_OK;
+}
+
 // Raises the dynamic shared-memory limit of every kernel of frame size F on the current device
 // (cudaFuncSetAttribute acts per device), once per device; thread-safe.
 template <int F>
@@ -90,6 +112,13 @@ int prepare_kernels() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_col_fwd_tma2<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColTma2<F>::smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_col_adj_tma2<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColTma2<F>::smem);
   }
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_fwd_p<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<F>::smem_row_fwd);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_fwd_p<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<F>::smem_row_fwd);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_col_fwd_p<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<F>::smem_col);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_col_adj_p<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<F>::smem_col);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_adj_p<F, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowAdjLSmemMax);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_adj_p<F, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowAdjLSmemMax);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_adj_p1<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, row_adj_p1_smem<F>());
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_rows<F, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowCfg<F>::smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_rows<F, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowCfg<F>::smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_rows<F, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowCfg<F>::smem);
@@ -129,7 +158,8 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
   // mode-summed object-gradient patch that the adjoint shift transforms)
   const bool shifted = p.d_delta != nullptr;
   if (shifted && (p.nchunks != 1 || !p.adj_l_ok)) return PTYCHO_EUNSUPPORTED;
-  const bool adj_l = (p.adj_l && !obj_atomic && p.nchunks == 1) || shifted;
+  const bool pair = p.pair != 0;                      // passes over pairs of positions
+  const bool adj_l = (p.adj_l && !obj_atomic && p.nchunks == 1) || shifted || pair;
   const bool col_staged = p.col_staged && p.nchunks == 1;
   const bool fwd_l = p.fwd_l && p.nchunks == 1 && !shifted;
   const bool narrow = (p.flags & PTYCHO_FLAG_NARROW_COLUMNS) != 0;
@@ -196,7 +226,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
   const int col_adj_smem = ColCfg<F>::smem_xch + F * ColCfg<F>::W * (int)sizeof(float);
   const int nbatches = (c.nbatch + p.B - 1) / p.B;
   const int nsets = p.nsets < nbatches ? p.nsets : nbatches;
-  const long long set_S = (long long)p.B * p.C * FF, set_I = (long long)p.B * a.G * FF, set_F = (long long)p.B * FF;
+  const long long set_S = (long long)(pair ? (p.B + 1) / 2 * 2 : p.B) * p.C * FF, set_I = (long long)p.B * a.G * FF, set_F = (long long)p.B * FF;
   cudaStream_t streams[ptycho_plan::kMaxSets] = {st};
   for (int i = 1; i < nsets; ++i) streams[i] = p.side[i - 1];
   if (nsets > 1) {                                    // the side streams follow the caller's work so far
@@ -272,6 +302,18 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
                                                 a, ct));
           continue;
         }
+      }
+      if (pair) {
+        const int np = (a.nb + 1) / 2;
+        auto* k_fwd = (reinterpret_cast<uintptr_t>(c.P) & 15) ? k_row_fwd_p<F, false> : k_row_fwd_p<F, true>;
+        // kRowFwdPairs pairs per block, fewer when that leaves under three waves of three blocks per SM
+        const int rows = F / PairCfg<F>::rows_fwd, want = (9 * p.sms + rows * p.L - 1) / (rows * p.L);
+        const int chunks = std::min(np, std::max(want, (np + kRowFwdPairs - 1) / kRowFwdPairs));
+        PTY_LAUNCH(p, kRowFwd, cs, launch_pdl(k_fwd, dim3(chunks, rows, p.L), 128, PairCfg<F>::smem_row_fwd, cs, c.O, c.P,
+                                              reinterpret_cast<float4*>(S), a));
+        PTY_LAUNCH(p, kColFwd, cs, launch_pdl(k_col_fwd_p<F>, dim3(F / PairCfg<F>::CW, p.G, np), PairCfg<F>::cthreads,
+                                              PairCfg<F>::smem_col, cs, p.tmap_pair[set], Ip, a));
+        continue;
       }
       bool warp_rows_fwd = false;
       if constexpr (F == 512) {
@@ -360,10 +402,15 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
           continue;
         }
       }
+      if (pair)
+        PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_col_adj_p<F>, dim3(F / PairCfg<F>::CW, p.G, (a.nb + 1) / 2),
+                                              PairCfg<F>::cthreads, PairCfg<F>::smem_col, cs, p.tmap_pair[set], a, aa));
       if (!store && rerun_rows)
         PTY_LAUNCH(p, kRowFwd, cs,
                    launch_pdl(k_row_fwd<F>, dim3(a.nb, F / RowCfg<F>::RPB, p.L), row_blk, RowCfg<F>::smem, cs, c.O, c.P, S, a));
-      if (col_staged) {
+      if (pair)
+        ;
+      else if (col_staged) {
         rc = narrow ? launch_cols_s<F, 4>(p, false, store, cs, S, Ip, a, aa) : launch_cols_s<F, 0>(p, false, store, cs, S, Ip, a, aa);
         if (rc) return rc;
       } else if (F == 512 && p.has_tma && p.col_tma2 && !store) {
@@ -390,8 +437,12 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
       if (adj_l) {
         constexpr int T = FftShape<F>::N1;
         bool warp_rows = false;
+        if (pair) {
+          rc = launch_row_adj_pair<F>(p, cs, c, S, gPs, a, nsplit);
+          if (rc) return rc;
+        }
         if constexpr (F == 512) {
-          if (p.adj_l_w) {
+          if (p.adj_l_w && !pair) {
             PTY_LAUNCH(p, kRowAdj, cs,
                        launch_pdl(k_row_adj_w<F>, dim3(F / p.rpb_adj, p.L, nsplit), 32 * p.M * p.rpb_adj,
                                   row_adj_w_smem(p.M, p.rpb_adj), cs, c.O, c.P, S, gPs, (long long)p.P_numel, a,
@@ -399,7 +450,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
             warp_rows = true;
           }
         }
-        if (warp_rows)
+        if (warp_rows || pair)
           ;
         else if (p.adj_l_pl2)
           PTY_LAUNCH(p, kRowAdj, cs,
@@ -414,19 +465,22 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
         if (nsets > 1 && cudaEventRecord(p.ev_radj[k % nsets], cs) != cudaSuccess) return PTYCHO_ECUDA;
         if (shifted) {                                // adjoint shift of the mode-summed patch gradients
           const dim3 rgrid(F / RowCfg<F>::RPB, p.L, a.nb), cgrid(F / ColCfg<F>::W, p.L, a.nb);
-          sh.src = S; sh.src_b = (long long)p.C * FF; sh.src_l = (long long)p.M * FF;
+          sh.src = S; sh.src_b = (long long)p.C * FF; sh.src_l = (long long)p.M * FF; sh.src_pair = pair;
           sh.dst = sh.T; sh.dst_b = (long long)p.L * FF; sh.dst_l = FF; sh.scale = 1.0f;
           PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_rows<F, false, false>, rgrid, row_blk, RowCfg<F>::smem, cs, c.O, a, sh));
           sh.dpart = c.g_delta ? p.d_dpart : nullptr;
           PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_cols<F, true>, cgrid, col_blk, ColCfg<F>::smem_xch, cs, a, sh));
-          sh.src = sh.T; sh.src_b = (long long)p.L * FF; sh.src_l = FF;
-          sh.dst = S; sh.dst_b = (long long)p.C * FF; sh.dst_l = (long long)p.M * FF; sh.scale = 1.0f / (float)FF;
+          sh.src = sh.T; sh.src_b = (long long)p.L * FF; sh.src_l = FF; sh.src_pair = 0;
+          sh.dst = S; sh.dst_b = (long long)p.C * FF; sh.dst_l = (long long)p.M * FF; sh.dst_pair = pair; sh.scale = 1.0f / (float)FF;
           PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_rows<F, true, false>, rgrid, row_blk, RowCfg<F>::smem, cs, c.O, a, sh));
           sh.dpart = nullptr;
         }
         if (nsets > 1 && k > 0 && cudaStreamWaitEvent(cs, p.ev_og[(k - 1) % nsets], 0) != cudaSuccess)
           return PTYCHO_ECUDA;
-        PTY_LAUNCH(p, kObjGrad, cs, launch_pdl(k_obj_grad_l<F>, dim3(max_tiles, p.L), 256, 0, cs, S, c.gO, a));
+        if (pair)
+          PTY_LAUNCH(p, kObjGrad, cs, launch_pdl(k_obj_grad_l<F, true>, dim3(max_tiles, p.L), 256, 0, cs, S, c.gO, a));
+        else
+          PTY_LAUNCH(p, kObjGrad, cs, launch_pdl(k_obj_grad_l<F, false>, dim3(max_tiles, p.L), 256, 0, cs, S, c.gO, a));
         if (nsets > 1 && cudaEventRecord(p.ev_og[k % nsets], cs) != cudaSuccess) return PTYCHO_ECUDA;
         continue;
       }

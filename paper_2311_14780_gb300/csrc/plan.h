@@ -41,6 +41,9 @@ struct ptycho_plan {
   int adj_l_w = 0;                             // F = 512: one warp per row (k_row_adj_w)
   int fwd_l_w = 0;                             // F = 512: one warp per row (k_row_fwd_w)
   int col_tma2 = 0;                            // F = 512: staged columns, half exchange, two blocks per SM
+  // passes over pairs of positions (pair.cuh): the default while all fields of a position fit; rows per
+  // block of their row adjoint (its position splits are nsplit_adj)
+  int pair = 0, rpb_pair = 1;
   // forward row pass over all modes of a wavelength per block (k_row_fwd_l), same rows per block
   int fwd_l = 0, nsplit_fwd = 1;
   // staged column passes (k_col_fwd_s / k_col_adj_s): one block per W columns of a position
@@ -104,6 +107,8 @@ struct ptycho_plan {
   // with a W x min(F, 256) box (column passes); has_tma = 0 falls back to plain loads
   int has_tma = 0;
   alignas(64) CUtensorMap tmap_S[4];
+  // pair passes: each scratch set as [pairs*C*F rows][4 F floats], boxes of one tile's columns
+  alignas(64) CUtensorMap tmap_pair[4];
   long long bytes = 0;
   long long last_launches = 0;
 

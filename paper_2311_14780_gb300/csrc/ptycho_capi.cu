@@ -8,6 +8,7 @@
 
 #include <cudaTypedefs.h>
 
+#include "pair.cuh"
 #include "plan.h"
 
 namespace ptycho {
@@ -375,6 +376,24 @@ void build_remap(int F, double z, double p, double alpha, std::vector<int32_t>& 
   }
 }
 
+// Sizes of the pair passes (pair.cuh) for frame size F: threads per vector, columns per tile, and the
+// shared memory of the row adjoint for M modes and rpb rows.
+struct PairSizes {
+  int T, CW, smem;
+};
+template <int F>
+PairSizes pair_sizes_of(int M, int rpb) {
+  return {ptycho::PairCfg<F>::T, ptycho::PairCfg<F>::CW, ptycho::row_adj_p_smem<F>(M, rpb)};
+}
+PairSizes pair_sizes(int F, int M, int rpb) {
+  switch (F) {
+    case 64: return pair_sizes_of<64>(M, rpb);
+    case 128: return pair_sizes_of<128>(M, rpb);
+    case 256: return pair_sizes_of<256>(M, rpb);
+    default: return pair_sizes_of<512>(M, rpb);
+  }
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link to libcuda).
 // Looked up once per process (a thread-safe static initialisation).
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
@@ -400,6 +419,20 @@ bool make_column_map(CUtensorMap* map, void* base, int F, long long rows, int W)
   const cuuint32_t estride[2] = {1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, base, dims, strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The same scratch for the pair passes: rows of 4 F floats, box of one tile (CW columns of 16 bytes),
+// swizzled as the column passes address it.
+bool make_pair_map(CUtensorMap* map, void* base, int F, long long rows, int CW) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+  if (!enc) return false;
+  const cuuint64_t dims[2] = {(cuuint64_t)F * 4, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)F * 16};
+  const cuuint32_t box[2] = {(cuuint32_t)(4 * CW), (cuuint32_t)(F < 256 ? F : 256)};
+  const cuuint32_t estride[2] = {1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CW == 8 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -543,6 +576,21 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
     p->C = (int)std::max<long long>(1, std::min<long long>(LM, p->scratch_budget / FF8));
     p->nchunks = (int)((LM + p->C - 1) / p->C);
   }
+  // passes over pairs of positions, unless a variant flag asks for the one-field passes
+  constexpr int kPairFlags = PTYCHO_FLAG_NO_PDL;
+  if (p->store && !g->zoom && !(g->flags & ~kPairFlags) && p->B >= 2 && LM >= 2) {
+    // rows per block of the row adjoint: whole warps of compute threads, and small blocks (64 compute
+    // threads) where the modes allow it, so that several are resident and drift apart
+    PairSizes z = pair_sizes(F, g->M, 1);
+    int rpb = 1;
+    while ((rpb * z.T * g->M) % 32) rpb *= 2;
+    while (2 * rpb * z.T * g->M <= 64 && 2 * rpb <= F) rpb *= 2;
+    if (g->M == 1 || (rpb * z.T * g->M <= ptycho::kRowAdjPairThreads && pair_sizes(F, g->M, rpb).smem <= ptycho::kRowAdjLSmemMax)) {
+      p->pair = 1;
+      p->rpb_pair = rpb;
+      if ((p->B & 1) && p->B < g->J) p->B += g->scratch_bytes > 0 || p->B == ptycho::kMaxB ? -1 : 1;
+    }
+  }
   int colblocks = 0;
   switch (F) {
     case 64: colblocks = F / ptycho::ColCfg<64>::W; break;
@@ -552,6 +600,11 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
   }
   const long long want_cols = 2ll * p->sms;   // column blocks wanted: mode groups only below two per SM
   long long G = (want_cols + (long long)colblocks * p->B - 1) / ((long long)colblocks * p->B);
+  if (p->pair) {                                      // and of the pair passes, in blocks of 128 threads
+    const PairSizes z = pair_sizes(F, g->M, 1);
+    const long long have = (long long)(F / z.CW) * ((p->B + 1) / 2) * z.CW * z.T / 128;
+    G = (want_cols + have - 1) / std::max<long long>(1, have);
+  }
   if (g->col_groups > 0) G = g->col_groups;
   G = std::max<long long>(1, std::min<long long>(G, p->C));
   p->MG = (int)((p->C + G - 1) / G);
@@ -608,6 +661,19 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
         ns = std::min<long long>(ns, std::min<long long>(64, p->B));
         while (ns > 1 && ns * p->P_numel * (long long)sizeof(float2) > (512ll << 20)) --ns;
         p->nsplit_adj = (int)std::max<long long>(1, ns);
+        if (p->pair) {
+          // (three waves of blocks; with one mode, six warps per SM)
+          const PairSizes z = pair_sizes(F, g->M, p->rpb_pair);
+          const int ct = z.T * g->M * p->rpb_pair;
+          const long long per_sm = std::max<long long>(1, std::min<long long>(12 / (ct / 32 + ptycho::row_adj_p_feeders(ct)),
+                                                                              (220 * 1024) / (z.smem + 8 * 1024)));
+          const long long blocks = g->M == 1 ? (long long)(F * z.T / 32) * g->L : (long long)(F / p->rpb_pair) * g->L;
+          const long long want = (g->M == 1 ? 6ll : 3ll * per_sm) * p->sms;
+          long long np = (want + blocks - 1) / blocks;
+          np = std::min<long long>(np, std::min<long long>(64, (p->B + 1) / 2));
+          while (np > 1 && np * p->P_numel * (long long)sizeof(float2) > (512ll << 20)) --np;
+          p->nsplit_adj = (int)std::max<long long>(1, np);
+        }
         // the forward row pass: same blocks, positions split for four blocks per SM.  Default at
         // 512^2 from 4 modes, where the probes of all modes outgrow the L2 and the fused pass reads
         // each probe row once per block instead of once per position: measured 153.4 vs 157.2 ms
@@ -681,7 +747,8 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
          cudaEventCreateWithFlags(&p->ev_join[i - 1], cudaEventDisableTiming) != cudaSuccess))
       rc = PTYCHO_ECUDA;
   }
-  rc = rc ? rc : dalloc(p, &p->d_S, (long long)p->nsets * p->B * p->C * FF);
+  const long long Bs = p->pair ? (p->B + 1) / 2 * 2 : p->B;   // positions of one scratch set (whole pairs)
+  rc = rc ? rc : dalloc(p, &p->d_S, (long long)p->nsets * Bs * p->C * FF);
   rc = rc ? rc : dalloc(p, &p->d_Ipart, (long long)p->nsets * p->B * std::max(p->G, p->res ? p->G_res : 1) * FF);
   rc = rc ? rc : dalloc(p, &p->d_D, (long long)p->nsets * p->B * FF);
   rc = rc ? rc : dalloc(p, &p->d_loss_part, (long long)g->J * (FF / (ptycho::kLossThreads * ptycho::kLossPx)));
@@ -715,9 +782,16 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
     p->has_tma = (g->flags & PTYCHO_FLAG_NO_TMA) || p->czt ? 0 : ((g->flags & PTYCHO_FLAG_TMA) || tma_default) ? 1 : 0;
     // F = 512: the staged column passes with the half-size exchange, two blocks per SM
     p->col_tma2 = F == 512 && !(g->flags & PTYCHO_FLAG_COLS_ONE_BLOCK) ? 1 : 0;
-    for (int i = 0; i < p->nsets; ++i)
+    if (p->pair) p->has_tma = 0;
+    for (int i = 0; i < p->nsets; ++i) {
       if (p->has_tma && !make_column_map(&p->tmap_S[i], p->d_S + (long long)i * p->B * p->C * FF, F, rows, W))
         p->has_tma = 0;
+      if (p->pair && !make_pair_map(&p->tmap_pair[i], p->d_S + (long long)i * Bs * p->C * FF, F, Bs / 2 * p->C * F,
+                                    pair_sizes(F, g->M, 1).CW)) {
+        free_plan(p);
+        return PTYCHO_ECUDA;
+      }
+    }
   }
 
   std::vector<int32_t> ident(g->J);

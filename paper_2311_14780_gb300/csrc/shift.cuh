@@ -34,12 +34,19 @@ struct ShiftArgs {
   long long src_b, src_l;        // element strides of the source between positions and wavelengths
   float2* dst;
   long long dst_b, dst_l;
+  int src_pair, dst_pair;        // the source or destination is a slot of the pair passes: positions 2p and
+                                 // 2p+1 share rows of 2 F values (2p first)
   float scale;                   // applied to the output (1 or 1/F^2)
   const float* delta;            // [L][J][2] fractional offsets (device)
   float2* T;                     // [B][L][F][F] transform workspace of the batch
   float2* Q;                     // [B][L][F][F] ramp * DFT2(window) of the batch
   double* dpart;                 // [nbatch][L][F/W][2] position-gradient partials, or null
 };
+
+// Offset of row r of the patch of (position b, wavelength l).
+__device__ __forceinline__ long long patch_row(int b, int l, int r, int F, long long sb, long long sl, int pair) {
+  return pair ? 2 * ((b >> 1) * sb + l * sl + (long long)r * F) + (b & 1) * F : b * sb + l * sl + (long long)r * F;
+}
 
 // Row DFT of the F x F patches of the batch, one row per T threads.
 // INV = false: source rows in natural order -> forward DFT -> destination in natural order;
@@ -59,8 +66,8 @@ k_shift_rows(const float2* __restrict__ O, KArgs a, ShiftArgs sa) {
   if (j < 0) return;                                  // uniform over the block
   const float2* src = FROM_O ? O + a.obj_off[l] + (long long)(a.pos[(l * a.J + j) * 2] + r) * a.obj_w[l] +
                                    a.pos[(l * a.J + j) * 2 + 1]
-                             : sa.src + b * sa.src_b + l * sa.src_l + (long long)r * F;
-  float2* dst = sa.dst + b * sa.dst_b + l * sa.dst_l + (long long)r * F;
+                             : sa.src + patch_row(b, l, r, F, sa.src_b, sa.src_l, sa.src_pair);
+  float2* dst = sa.dst + patch_row(b, l, r, F, sa.dst_b, sa.dst_l, sa.dst_pair);
   float2* xc = smem + vec * Xch<F>::region_rows;
   float2 v[N2];
   if (!INV) {
