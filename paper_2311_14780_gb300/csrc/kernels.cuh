@@ -1527,11 +1527,12 @@ __global__ void k_sum_splits(const float2* __restrict__ part, int nsplit, long l
 
 // ---------------------------------------------------------------------------------------
 // object gradient from one mode-summed slot per (position, wavelength) (after k_row_adj_l):
-// one block per 32x32 tile of grad O_l inside the batch's bounding box.  The positions whose
-// patches overlap the tile are listed first (ascending), then added four at a time with
-// their loads issued together.   grid (tiles of the largest box, L)
+// one block per tile (32 columns, 8 KR rows) of grad O_l inside the batch's bounding box.  The positions
+// whose patches overlap the tile are listed first (ascending), then added in groups with
+// their loads issued together: 16 / KR patches of KR rows per thread.  KR = 4 unless that leaves SMs
+// idle (k_obj_grad_l's launch).   grid (tiles of the largest box, L)
 // ---------------------------------------------------------------------------------------
-template <int F, bool PAIR = false>
+template <int F, bool PAIR = false, int KR = 4>
 __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, float2* __restrict__ gO, const KArgs& a,
                                                 const uint3 bid) {
   __shared__ int2 spos[kMaxB];
@@ -1541,10 +1542,11 @@ __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, fl
   const int l = bid.y;
   const int by0 = a.box[l][0], bx0 = a.box[l][1];
   const int ntx = (a.box[l][3] - bx0 + kTile - 1) / kTile;
-  const int nty = (a.box[l][2] - by0 + kTile - 1) / kTile;
+  constexpr int TH = 8 * KR;                          // tile height
+  const int nty = (a.box[l][2] - by0 + TH - 1) / TH;
   if ((int)bid.x >= ntx * nty) return;          // uniform over the block
   stage_batch(a, l, spos, ssig);
-  const int oy0 = by0 + ((int)bid.x / ntx) * kTile, ox0 = bx0 + ((int)bid.x % ntx) * kTile;
+  const int oy0 = by0 + ((int)bid.x / ntx) * TH, ox0 = bx0 + ((int)bid.x % ntx) * kTile;
   if (threadIdx.x < 32) {                             // ordered compaction by warp 0
     int n = 0;
     for (int b0 = 0; b0 < a.nb; b0 += 32) {
@@ -1552,7 +1554,7 @@ __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, fl
       bool hit = false;
       if (b < a.nb) {
         const int y = spos[b].x, x = spos[b].y;
-        hit = !(y < 0 || y >= oy0 + kTile || y + F <= oy0 || x >= ox0 + kTile || x + F <= ox0);
+        hit = !(y < 0 || y >= oy0 + TH || y + F <= oy0 || x >= ox0 + kTile || x + F <= ox0);
       }
       const unsigned mask = __ballot_sync(0xffffffffu, hit);
       if (hit) list[n + __popc(mask & ((1u << threadIdx.x) - 1u))] = b;
@@ -1566,12 +1568,12 @@ __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, fl
   const int tx = threadIdx.x % kTile, ty0 = threadIdx.x / kTile;   // 8 row slots
   const int ox = ox0 + tx;
   const int slot0 = l * a.M - a.chunk_base;
-  float2 acc[kTile / 8];
+  float2 acc[KR];
 #pragma unroll
-  for (int k = 0; k < kTile / 8; ++k) acc[k] = make_float2(0.f, 0.f);
-  constexpr int PG = 4;                               // patches per group of loads
+  for (int k = 0; k < KR; ++k) acc[k] = make_float2(0.f, 0.f);
+  constexpr int PG = 16 / KR;                         // patches per group of loads
   for (int i0 = 0; i0 < n; i0 += PG) {
-    float2 v[PG][kTile / 8];
+    float2 v[PG][KR];
 #pragma unroll
     for (int pp = 0; pp < PG; ++pp) {
       const int b = i0 + pp < n ? list[i0 + pp] : -1;
@@ -1581,7 +1583,7 @@ __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, fl
       const float2* src = PAIR ? S + ((long long)(bs >> 1) * a.C + slot0) * 2 * F * F + (bs & 1) * F + (ox - x)
                                : S + ((long long)bs * a.C + slot0) * F * F + (ox - x);
 #pragma unroll
-      for (int k = 0; k < kTile / 8; ++k) {
+      for (int k = 0; k < KR; ++k) {
         const int oy = oy0 + ty0 + 8 * k;
         const bool ok = in_x && oy >= y && oy < y + F;
         v[pp][k] = ok ? src[(long long)(oy - y) * (PAIR ? 2 * F : F)] : make_float2(0.f, 0.f);
@@ -1590,11 +1592,11 @@ __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, fl
 #pragma unroll
     for (int pp = 0; pp < PG; ++pp)
 #pragma unroll
-      for (int k = 0; k < kTile / 8; ++k) acc[k] = cadd(acc[k], v[pp][k]);
+      for (int k = 0; k < KR; ++k) acc[k] = cadd(acc[k], v[pp][k]);
   }
   float2* g = gO + a.obj_off[l];
 #pragma unroll
-  for (int k = 0; k < kTile / 8; ++k) {
+  for (int k = 0; k < KR; ++k) {
     const int oy = oy0 + ty0 + 8 * k;
     if (oy < H && ox < Wd) {
       float2* p = g + (long long)oy * Wd + ox;
@@ -1604,18 +1606,57 @@ __device__ __forceinline__ void obj_grad_l_body(const float2* __restrict__ S, fl
 }
 
 // PAIR: the slots of the pair passes (rows of 2 F float2: lane 0's row, then lane 1's).
-template <int F, bool PAIR>
+template <int F, bool PAIR, int KR>
 __global__ void __launch_bounds__(256)
 k_obj_grad_l(const float2* __restrict__ S, float2* __restrict__ gO, KArgs a) {
   pdl_wait();
   pdl_trigger();
-  obj_grad_l_body<F, PAIR>(S, gO, a, blockIdx);
+  obj_grad_l_body<F, PAIR, KR>(S, gO, a, blockIdx);
+}
+
+// ---------------------------------------------------------------------------------------
+// fixed-order sums
+// ---------------------------------------------------------------------------------------
+constexpr int kReduceThreads = 256, kReduceBlocks = 8;
+__device__ __forceinline__ double warp_sum(double s) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+// Sum over i = first, first + stride, ... < n of part[i], over a block of kReduceThreads threads; valid in
+// thread 0.
+__device__ __forceinline__ double block_sum_partials(const double* __restrict__ part, long long n, int first, int stride,
+                                                     double* red) {
+  constexpr int U = 4;
+  double s[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) s[u] = 0.0;
+  long long i = first;
+  for (; i + (U - 1) * stride < n; i += U * stride)
+#pragma unroll
+    for (int u = 0; u < U; ++u) s[u] += part[i + u * stride];
+  for (; i < n; i += stride) s[0] += part[i];
+  const double v = warp_sum((s[0] + s[1]) + (s[2] + s[3]));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < kReduceThreads / 32; ++w) t += red[w];
+  return t;
+}
+// f(i) by a whole warp for every call entry i with bidx[i] = j, in order.
+template <class Fn>
+__device__ __forceinline__ void for_entries_of(const int32_t* __restrict__ bidx, int nbatch, int j, int lane, Fn&& f) {
+  for (int i0 = 0; i0 < nbatch; i0 += 32) {
+    unsigned hit = __ballot_sync(0xffffffffu, i0 + lane < nbatch && __ldg(bidx + i0 + lane) == j);
+    for (; hit; hit &= hit - 1) f(i0 + __ffs(hit) - 1);
+  }
 }
 
 // ---------------------------------------------------------------------------------------
 // loss reduction and Adam (defined in ptycho_capi.cu)
 // ---------------------------------------------------------------------------------------
-__global__ void k_loss_reduce(const double* __restrict__ part, long long n, double* out);
+__global__ void k_loss_reduce(const double* __restrict__ part, long long n, double* out);   // grid kReduceBlocks
 __global__ void k_sigma_grad(const int32_t* __restrict__ bidx, int nbatch, int J, const double* __restrict__ part,
                              int nblk, const float* __restrict__ sigma, float* __restrict__ g);
 __global__ void k_sum_sets(const float* __restrict__ acc, int nsets, long long n, float* __restrict__ out);

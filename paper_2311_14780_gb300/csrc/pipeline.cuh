@@ -22,6 +22,12 @@ namespace ptycho {
     prof_end((p), pty_ev, (st));                                     \
   } while (0)
 
+// 32 x 32 tiles of the object gradient per SM below which it takes 8-row tiles (a tile adds its patches one
+// group after another: 400 positions of 128^2 on a 400^2 object, 169 tiles: 25 us with 8 rows; with three
+// batches of 134 and 32 rows 76 us in all)
+constexpr int kObjGradBlocksPerSM = 2;
+
+
 template <int F, int WN>
 cudaError_t set_cols_smem() {
   cudaError_t e = cudaFuncSetAttribute(k_col_fwd_s<F, true, WN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -248,7 +254,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
     a.nb = (c.nbatch - off < p.B) ? (c.nbatch - off) : p.B;
     // region of each object the batch's patches cover (exact for the identity order, else
     // the whole object); the object-gradient kernel tiles it
-    int max_tiles = 1;
+    int max_tiles = 1, max_tiles8 = 1;                // of 32 x 32 and of 8 x 32 (rows x columns)
     for (int l = 0; l < p.L && grad; ++l) {
       int y0 = 0, x0 = 0, y1 = p.obj_h[l], x1 = p.obj_w[l];
       if (identity) {
@@ -263,6 +269,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
       a.box[l][0] = y0; a.box[l][1] = x0; a.box[l][2] = y1; a.box[l][3] = x1;
       const int tiles = ((y1 - y0 + kTile - 1) / kTile) * ((x1 - x0 + kTile - 1) / kTile);
       max_tiles = tiles > max_tiles ? tiles : max_tiles;
+      max_tiles8 = std::max(max_tiles8, ((y1 - y0 + 7) / 8) * ((x1 - x0 + kTile - 1) / kTile));
     }
     // forward: all chunks accumulate the model intensity
     // fractional offsets: shift the batch's object windows into the patch buffer
@@ -477,10 +484,12 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
         }
         if (nsets > 1 && k > 0 && cudaStreamWaitEvent(cs, p.ev_og[(k - 1) % nsets], 0) != cudaSuccess)
           return PTYCHO_ECUDA;
-        if (pair)
-          PTY_LAUNCH(p, kObjGrad, cs, launch_pdl(k_obj_grad_l<F, true>, dim3(max_tiles, p.L), 256, 0, cs, S, c.gO, a));
-        else
-          PTY_LAUNCH(p, kObjGrad, cs, launch_pdl(k_obj_grad_l<F, false>, dim3(max_tiles, p.L), 256, 0, cs, S, c.gO, a));
+        // 32 x 32 tiles, or 32 x 8 when fewer than kObjGradBlocks of the former would run: each block adds
+        // its overlapping patches one group after another, and few blocks are bound by that chain
+        const bool small = max_tiles * p.L < kObjGradBlocksPerSM * p.sms;
+        auto* k_og = pair ? (small ? k_obj_grad_l<F, true, 1> : k_obj_grad_l<F, true, 4>)
+                          : (small ? k_obj_grad_l<F, false, 1> : k_obj_grad_l<F, false, 4>);
+        PTY_LAUNCH(p, kObjGrad, cs, launch_pdl(k_og, dim3(small ? max_tiles8 : max_tiles, p.L), 256, 0, cs, S, c.gO, a));
         if (nsets > 1 && cudaEventRecord(p.ev_og[k % nsets], cs) != cudaSuccess) return PTYCHO_ECUDA;
         continue;
       }
@@ -508,15 +517,15 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
                launch_pdl(k_sum_splits, dim3(4 * p.sms), 256, 0, st, (const float2*)gPs, nsplit, p.P_numel, c.gP));
   if (grad && c.g_z)
     PTY_LAUNCH(p, kLossReduce, st,
-               launch_pdl(k_loss_reduce, 1, 256, 0, st, (const double*)p.d_z_part,
+               launch_pdl(k_loss_reduce, kReduceBlocks, kReduceThreads, 0, st, (const double*)p.d_z_part,
                           (long long)c.nbatch * loss_blocks<F>(), c.g_z));
   if (grad && c.g_delta)
     PTY_LAUNCH(p, kShift, st,
-               launch_pdl(k_delta_grad, dim3((p.L * p.J + 255) / 256), 256, 0, st, (const int32_t*)c.bidx, c.nbatch,
+               launch_pdl(k_delta_grad, dim3((p.L * p.J + 7) / 8), 256, 0, st, (const int32_t*)c.bidx, c.nbatch,
                           p.L, p.J, (const double*)p.d_dpart, F / ColCfg<F>::W, c.g_delta));
   if (grad && c.g_sigma)
     PTY_LAUNCH(p, kLossReduce, st,
-               launch_pdl(k_sigma_grad, dim3((p.J + 255) / 256), 256, 0, st, (const int32_t*)c.bidx, c.nbatch, p.J,
+               launch_pdl(k_sigma_grad, dim3((p.J + 7) / 8), 256, 0, st, (const int32_t*)c.bidx, c.nbatch, p.J,
                           (const double*)p.d_sig_part, loss_blocks<F>(), c.sigma, c.g_sigma));
   if (grad && c.g_bg)
     PTY_LAUNCH(p, kLossReduce, st,
@@ -526,7 +535,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
     double* out = c.loss;
     if (out) {
       PTY_LAUNCH(p, kLossReduce, st,
-                 launch_pdl(k_loss_reduce, 1, 256, 0, st, p.d_loss_part, (long long)c.nbatch * loss_blocks<F>(), out));
+                 launch_pdl(k_loss_reduce, kReduceBlocks, kReduceThreads, 0, st, p.d_loss_part, (long long)c.nbatch * loss_blocks<F>(), out));
     }
   }
   return PTYCHO_OK;

@@ -196,7 +196,7 @@ int plain_adjoint(ptycho_plan& p, const CallArgs& c, float2* psi, float* Ibuf, f
   }
   if (c.loss) {
     PTY_LAUNCH(p, kLossReduce, st,
-               k_loss_reduce<<<1, 256, 0, st>>>(p.d_loss_part, (long long)c.nbatch * loss_blocks<F>(), c.loss));
+               k_loss_reduce<<<kReduceBlocks, kReduceThreads, 0, st>>>(p.d_loss_part, (long long)c.nbatch * loss_blocks<F>(), c.loss));
   }
   return PTYCHO_OK;
 }

@@ -6,6 +6,7 @@
 #include <new>
 #include <vector>
 
+#include <cooperative_groups.h>
 #include <cudaTypedefs.h>
 
 #include "pair.cuh"
@@ -13,69 +14,89 @@
 
 namespace ptycho {
 
-// Fixed-order FP64 sum of the per-block loss partials (one block).
-__global__ void __launch_bounds__(256) k_loss_reduce(const double* __restrict__ part, long long n, double* out) {
+// Fixed-order FP64 sum of the per-block loss partials: one cluster of kReduceBlocks blocks, whose sums the
+// first block adds in block order through distributed shared memory.  FP64 additions bound it (two per
+// clock and SM on this part), so it wants several SMs: 102 400 partials (400 frames of 512^2) took 49 us
+// in one block of 256 threads, 36 us in one of 1024.
+__global__ void __cluster_dims__(kReduceBlocks, 1, 1) __launch_bounds__(kReduceThreads)
+k_loss_reduce(const double* __restrict__ part, long long n, double* out) {
   pdl_wait();
-  __shared__ double red[256];
-  double s = 0.0;
-  for (long long i = threadIdx.x; i < n; i += 256) s += part[i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  __shared__ double red[kReduceThreads / 32];
+  __shared__ double sums[kReduceBlocks];
+  const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int rank = (int)cl.block_rank();
+  const double s = block_sum_partials(part, n, rank * kReduceThreads + (int)threadIdx.x, kReduceBlocks * kReduceThreads, red);
+  if (threadIdx.x == 0) *cl.map_shared_rank(&sums[rank], 0) = s;
+  cl.sync();
+  if (rank == 0 && threadIdx.x == 0) {
+    double t = 0.0;
+    for (int k = 0; k < kReduceBlocks; ++k) t += sums[k];
+    *out = t;
   }
-  if (threadIdx.x == 0) *out = red[0];
 }
 
 // Gradient of the power coefficients.  sigma_j multiplies every exit wave of frame j (f1),
 // and the DFT is unitary, so sum_r conj(psi) chi = 2 sum_k G_k |Psi_k|^2 and
 // dL/dsigma_j = (2 / sigma_j) sum over the camera grid of D * (R sum_lm |Psi_lm|^2), the
-// quantity the loss kernel left per block in part.  One thread per position j sums, in
-// entry order, the partials of every call entry i with bidx[i] = j; positions outside the
-// call (and sigma_j = 0, where the derivative vanishes) get 0.
+// quantity the loss kernel left per block in part.  One warp per position j walks the call's
+// entries in order and adds the partials of every entry i with bidx[i] = j (lanes stride over an entry's
+// partials, then a fixed tree); positions outside the call (and sigma_j = 0, where the derivative
+// vanishes) get 0.  One thread per position took 189 us for 400 entries of 64 partials: a serial chain
+// over the entries, each with a dependent load.
 __global__ void __launch_bounds__(256)
 k_sigma_grad(const int32_t* __restrict__ bidx, int nbatch, int J, const double* __restrict__ part, int nblk,
              const float* __restrict__ sigma, float* __restrict__ g) {
   pdl_wait();
-  const int j = blockIdx.x * 256 + threadIdx.x;
-  if (j >= J) return;
+  const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (j >= J) return;                                 // uniform over the warp
   double s = 0.0;
-  for (int i = 0; i < nbatch; ++i) {
-    if (__ldg(bidx + i) != j) continue;
-    for (int k = 0; k < nblk; ++k) s += part[(long long)i * nblk + k];
-  }
+  for_entries_of(bidx, nbatch, j, lane, [&](int i) {
+    for (int k = lane; k < nblk; k += 32) s += part[(long long)i * nblk + k];
+  });
+  s = warp_sum(s);
   const float sj = sigma ? __ldg(sigma + j) : 1.0f;
-  g[j] = sj != 0.f ? (float)(2.0 * s / (double)sj) : 0.f;
+  if (lane == 0) g[j] = sj != 0.f ? (float)(2.0 * s / (double)sj) : 0.f;
 }
 
+// Position gradient, one warp per (l, j) in the same way (one thread each: 112 us for 400 entries).
 __global__ void __launch_bounds__(256)
 k_delta_grad(const int32_t* __restrict__ bidx, int nbatch, int L, int J, const double* __restrict__ dpart,
              int nstrips, float* __restrict__ g_delta) {
   pdl_wait();
-  const int e = blockIdx.x * 256 + threadIdx.x;       // e = l*J + j
+  const int e = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;   // e = l*J + j
   if (e >= L * J) return;
   const int l = e / J, j = e % J;
   double sy = 0.0, sx = 0.0;
-  for (int i = 0; i < nbatch; ++i) {
-    if (__ldg(bidx + i) != j) continue;
+  for_entries_of(bidx, nbatch, j, lane, [&](int i) {
     const double* d = dpart + ((long long)i * L + l) * nstrips * 2;
-    for (int k = 0; k < nstrips; ++k) {
+    for (int k = lane; k < nstrips; k += 32) {
       sy += d[2 * k];
       sx += d[2 * k + 1];
     }
+  });
+  sy = warp_sum(sy);
+  sx = warp_sum(sx);
+  if (lane == 0) {
+    g_delta[2 * e] = (float)sy;
+    g_delta[2 * e + 1] = (float)sx;
   }
-  g_delta[2 * e] = (float)sy;
-  g_delta[2 * e + 1] = (float)sx;
 }
 
-// out[i] = sum over the probe-gradient splits, in split order, of part[s][i].
+// out[i] = sum over the probe-gradient splits, in split order, of part[s][i] (eight loads in flight).
 __global__ void __launch_bounds__(256)
 k_sum_splits(const float2* __restrict__ part, int nsplit, long long n, float2* __restrict__ out) {
   pdl_wait();
   for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
     float2 s = part[i];
-    for (int k = 1; k < nsplit; ++k) s = cadd(s, part[(long long)k * n + i]);
+    int k = 1;
+    for (; k + 8 <= nsplit; k += 8) {
+      float2 v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = part[(long long)(k + q) * n + i];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s = cadd(s, v[q]);
+    }
+    for (; k < nsplit; ++k) s = cadd(s, part[(long long)k * n + i]);
     out[i] = s;
   }
 }
@@ -154,17 +175,25 @@ using ptycho::CallKind;
 
 namespace {
 
-// The default batching: about kBatchEvals evaluations per batch, but at least kMinBatchPositions
-// positions, one buffer set of at most kMaxScratch.  Measured on 512^2 x 6 wavelengths x 10
-// modes (120 MB of fields per position), where the per-batch work that does not grow with the
-// batch (reading the probes in the forward and adjoint rows, adding into the probe gradient,
-// the launches' tails) is largest: 17 / 20 / 26 / 34 / 45 / 60 / 75 / 100 positions per batch
-// gave 143.0 / 141.5 / 140.3 / 138.7 / 137.0 / 136.1 / 135.6 / 134.8 ms per step (three batches
-// in flight); 512^2 x 8 modes x 5 wavelengths: 41.8 ms with 25 positions, 40.9 with 58.
+// The default batching: about kBatchElems field elements per batch, but at least kMinBatchPositions
+// positions, one buffer set of at most kMaxScratch, and up to kMinBatches batches per call (they overlap)
+// as long as each holds kSmallBatchElems.
+//
+// Large fields: measured on 512^2 x 6 wavelengths x 10 modes (120 MB of fields per position), where the
+// per-batch work that does not grow with the batch (reading the probes in the forward and adjoint
+// rows, adding into the probe gradient, the launches' tails) is largest: 17 / 20 / 26 / 34 / 45 /
+// 60 / 75 / 100 positions per batch gave 143.0 / 141.5 / 140.3 / 138.7 / 137.0 / 136.1 / 135.6 / 134.8 ms
+// per step with the one-field passes; with the pair passes 30 / 60 / 100 gave 125.6 / 121.7 / 120.8.
+// Small frames want more evaluations per launch than the 1200 that 512^2 wants: 128^2 x 8 modes x 5
+// wavelengths with 32 / 58 / 80 / 134 positions per batch (400 in all) 2.48 / 2.29 / 2.28 / 2.13 ms,
+// 256^2 x 4 x 3 with 50 / 68 / 100 / 134 3.18 / 3.13 / 3.06 / 3.00 ms: so the target is in elements.
+// One field per position: 64^2 with 22 / 32 / 64 of 64 positions 139 / 117 / 98 us (launches), 128^2
+// with 68 / 134 / 200 / 400 of 400 positions 262 / 243 / 235 / 241 us.
 constexpr long long kMaxScratch = 8ll << 30;   // default upper bound of one buffer set
-constexpr long long kBatchEvals = 1200;        // evaluations per batch the default aims for
-constexpr long long kMinBatchPositions = 64;   // and at least this many positions (when they fit)
-constexpr long long kMinBatches = 3;           // and at least this many batches per call (overlap)
+constexpr long long kBatchElems = 320ll << 20; // field elements per batch the default aims for (1200 of 512^2)
+constexpr long long kSmallBatchElems = 4ll << 20;
+constexpr long long kMinBatchPositions = 64;   // at least this many positions (when they fit)
+constexpr long long kMinBatches = 3;           // batches per call (overlap), when they are not small
 constexpr long long kBatchRows = 32768;        // and at least this many 1D FFT rows per pass
 constexpr int kDefaultOverlap = 3;             // position batches in flight
 constexpr double kPi = 3.14159265358979323846;
@@ -484,7 +513,7 @@ const char* ptycho_strerror(int code) {
 }
 
 int ptycho_plan_create(const ptycho_geom_t* g, ptycho_plan_t** out) {
-  return ptycho::create_plan(g, ptycho::BatchTarget{kBatchEvals, kMinBatchPositions, kMaxScratch}, out);
+  return ptycho::create_plan(g, ptycho::BatchTarget{0, kBatchElems, kMinBatchPositions, kMaxScratch}, out);
 }
 
 }  // extern "C"
@@ -545,7 +574,7 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
   p->pos_host.assign(g->pos, g->pos + (size_t)g->L * g->J * 2);
 
   // batching: a batch keeps the fields of all L*M modes of B positions in the scratch (store
-  // mode, no recompute) with B chosen so that one launch carries about kBatchEvals
+  // mode, no recompute) with B chosen so that one launch carries about the target's
   // evaluations; a small scratch stays in L2, a large one spills to HBM, which costs less than
   // launching small batches.  Only when one position's fields exceed the budget are the modes
   // split into chunks that the adjoint recomputes (small-mode problems also get at least
@@ -560,9 +589,12 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
     p->nchunks = 1;
     long long B = p->scratch_budget / (LM * FF8);
     if (g->scratch_bytes <= 0) {
-      B = std::min<long long>(B, std::max({(target.evals + LM - 1) / LM, (kBatchRows + LM * F - 1) / (LM * F),
+      const long long elems = LM * F * F;               // of one position
+      const long long evals = std::max(target.evals, (target.elems + F * F - 1) / (F * F));
+      B = std::min<long long>(B, std::max({(evals + LM - 1) / LM, (kBatchRows + LM * F - 1) / (LM * F),
                                            target.min_positions}));
-      B = std::min<long long>(B, std::max<long long>(1, (g->J + kMinBatches - 1) / kMinBatches));
+      const long long nmin = std::max<long long>(1, std::min<long long>(kMinBatches, g->J * elems / kSmallBatchElems));
+      B = std::min<long long>(B, std::max<long long>(1, (g->J + nmin - 1) / nmin));
     }
     p->B = (int)std::max<long long>(1, std::min<long long>(B, ptycho::kMaxB));
     p->B = std::min(p->B, g->J);
@@ -576,9 +608,12 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
     p->C = (int)std::max<long long>(1, std::min<long long>(LM, p->scratch_budget / FF8));
     p->nchunks = (int)((LM + p->C - 1) / p->C);
   }
-  // passes over pairs of positions, unless a variant flag asks for the one-field passes
+  // passes over pairs of positions, unless a variant flag asks for the one-field passes.  With one field
+  // per position a column tile has no second mode to fetch meanwhile: at 512^2 the one-field column passes
+  // are the faster ones (400 positions: 3.22 vs 3.54 ms per step), at 128^2 the pair passes (246 vs 256 us;
+  // at 64^2 both wait for the launches)
   constexpr int kPairFlags = PTYCHO_FLAG_NO_PDL;
-  if (p->store && !g->zoom && !(g->flags & ~kPairFlags) && p->B >= 2 && LM >= 2) {
+  if (p->store && !g->zoom && !(g->flags & ~kPairFlags) && p->B >= 2 && (LM >= 2 || F <= 128)) {
     // rows per block of the row adjoint: whole warps of compute threads, and small blocks (64 compute
     // threads) where the modes allow it, so that several are resident and drift apart
     PairSizes z = pair_sizes(F, g->M, 1);

@@ -46,18 +46,11 @@ extern template cudaError_t prepare_multi<512>();
 namespace ptycho {
 
 // One block per site: fixed-order FP64 sum of its loss partials.
-__global__ void __launch_bounds__(256) k_loss_reduce_multi(const SiteFinish* __restrict__ sf) {
-  __shared__ double red[256];
+__global__ void __launch_bounds__(kReduceThreads) k_loss_reduce_multi(const SiteFinish* __restrict__ sf) {
+  __shared__ double red[kReduceThreads / 32];
   const SiteFinish& f = sf[blockIdx.x];
-  double s = 0.0;
-  for (long long i = threadIdx.x; i < f.nparts; i += 256) s += f.loss_part[i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *f.loss = red[0];
+  const double s = block_sum_partials(f.loss_part, f.nparts, (int)threadIdx.x, kReduceThreads, red);
+  if (threadIdx.x == 0) *f.loss = s;
 }
 
 // The fused row adjoint's probe-gradient splits of every site that has several, added in split
@@ -405,7 +398,7 @@ int enqueue_shared_tick(const std::vector<Site*>& sites, const TickTables& tt, c
     if (rc) return rc;
   }
   if (splits) ptycho::k_sum_splits_multi<<<dim3(tt.adam_blocks, tt.nsites), 256, 0, st>>>(tt.finish);
-  ptycho::k_loss_reduce_multi<<<tt.nsites, 256, 0, st>>>(tt.finish);
+  ptycho::k_loss_reduce_multi<<<tt.nsites, ptycho::kReduceThreads, 0, st>>>(tt.finish);
   ptycho::k_tick_multi<<<(tt.nsites + 255) / 256, 256, 0, st>>>(tt.finish, tt.nsites);
   ptycho::k_adam_multi<<<dim3(tt.adam_blocks, 2 * tt.nsites), 256, 0, st>>>(tt.finish);
   return cudaGetLastError() == cudaSuccess ? PTYCHO_OK : PTYCHO_ECUDA;
