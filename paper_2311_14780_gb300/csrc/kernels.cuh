@@ -32,6 +32,13 @@ constexpr int kMaxL = 16;
 constexpr int kLossThreads = 256;
 constexpr int kLossPx = 4;       // camera pixels per thread in the loss kernel (a multiple of 4)
 template <int F> __host__ __device__ constexpr int loss_blocks() { return F * F / (kLossThreads * kLossPx); }
+constexpr int kLossPosMax = 8;   // positions per block of the loss kernel, at most
+// Positions per block: as many as leave four blocks per SM.
+inline int loss_positions(int F, int nb, int sms) {
+  int np = kLossPosMax;
+  while (np > 1 && (long long)(F * F / (kLossThreads * kLossPx)) * ((nb + np - 1) / np) < 4ll * sms) np /= 2;
+  return np;
+}
 constexpr int kTile = 32;        // object-gradient tile side
 constexpr int kMaxB = 512;       // positions per batch (upper bound)
 
@@ -417,6 +424,7 @@ struct LossArgs {
   float* I_pred;                 // [J][F][F] or null
   int remap;
   int Gsum;                      // intensity slices (mode groups) to add
+  int npos;                      // positions per block (1 to kLossPosMax)
   const float2* tap_dz;          // [F*F] d(row, col index of the taps)/dz (remap only)
   double* z_part;                // [nbatch][loss_blocks] sums of D * d(R I)/dz, or null
 };
@@ -456,46 +464,9 @@ __device__ __forceinline__ float poisson_term(float Ie, float Ih) {
   return Ih * f;
 }
 
-// Camera-grid prediction of one pixel q (remap: bilinear in the four model taps of q).
-// Is is the field part, Ib the background part; valid = false outside the remap's grid.
-// With the remap, srow / scol are the slopes of the bilinear interpolant of the full model
-// intensity (field + background) along the row and column fractions of the taps.
-template <int F>
-__device__ __forceinline__ void predict_pixel(const LossArgs& la, const float* Ip, int G, int q, int tb, float2 w,
-                                              float& Is, float& Ib, bool& valid, float& srow, float& scol) {
-  constexpr int FF = F * F;
-  Is = 0.f;
-  Ib = 0.f;
-  srow = scol = 0.f;
-  valid = true;
-  if (la.remap) {
-    valid = tb >= 0;
-    if (!valid) return;
-    float i00, i01, i10, i11;
-    if (G == 1) {                                     // one intensity slice (uniform branch)
-      i00 = Ip[tb];
-      i01 = Ip[tb + 1];
-      i10 = Ip[tb + F];
-      i11 = Ip[tb + F + 1];
-    } else {
-      i00 = model_I(Ip, G, FF, tb);
-      i01 = model_I(Ip, G, FF, tb + 1);
-      i10 = model_I(Ip, G, FF, tb + F);
-      i11 = model_I(Ip, G, FF, tb + F + 1);
-    }
-    Is = (1.f - w.x) * ((1.f - w.y) * i00 + w.y * i01) + w.x * ((1.f - w.y) * i10 + w.y * i11);
-    if (la.bg) {
-      const float b00 = __ldg(la.bg + tb), b01 = __ldg(la.bg + tb + 1);
-      const float b10 = __ldg(la.bg + tb + F), b11 = __ldg(la.bg + tb + F + 1);
-      Ib = (1.f - w.x) * ((1.f - w.y) * b00 + w.y * b01) + w.x * ((1.f - w.y) * b10 + w.y * b11);
-      i00 += b00; i01 += b01; i10 += b10; i11 += b11;
-    }
-    srow = ((1.f - w.y) * i10 + w.y * i11) - ((1.f - w.y) * i00 + w.y * i01);
-    scol = (1.f - w.x) * (i01 - i00) + w.x * (i11 - i10);
-  } else {
-    Is = model_I(Ip, G, FF, q);
-    if (la.bg) Ib = __ldg(la.bg + q);
-  }
+// Bilinear value of the four taps i00, i01 (row), i10, i11 (row + 1) with weights w = (row, column).
+__device__ __forceinline__ float bilinear(float2 w, float i00, float i01, float i10, float i11) {
+  return (1.f - w.x) * ((1.f - w.y) * i00 + w.y * i01) + w.x * ((1.f - w.y) * i10 + w.y * i11);
 }
 
 // Compensated FP32 sums ("double-float": value = hi + lo).  Knuth's TwoSum gives the exact
@@ -528,111 +499,180 @@ __device__ __forceinline__ void df_warp_sum(float& hi, float& lo) {
   }
 }
 
-// Each thread takes kLossPx consecutive camera pixels; the loss terms and the sigma-gradient
-// terms of a block are summed as double-floats (per thread, then a warp tree) and the eight
-// warp sums in FP64, in a fixed order, into one partial per (call entry, block).
-// grid (F*F/(kLossThreads*kLossPx), nb)
-template <int F>
-__device__ __forceinline__ void loss_body(const KArgs& a, const LossArgs& la, const uint3 bid) {
-  constexpr int FF = F * F, NB = loss_blocks<F>();
-  __shared__ float red[6][kLossThreads / 32];
-  const int b = bid.y;
-  const int i = a.batch_off + b;
-  const int q0 = (bid.x * kLossThreads + threadIdx.x) * kLossPx;
-  const int j = batch_pos(a, i);                     // uniform over the block
-  if (j < 0) {
-    if (la.loss_part && threadIdx.x == 0) la.loss_part[(long long)i * NB + bid.x] = 0.0;
-    if (la.sig_part && threadIdx.x == 0) la.sig_part[(long long)i * NB + bid.x] = 0.0;
-    if (la.z_part && threadIdx.x == 0) la.z_part[(long long)i * NB + bid.x] = 0.0;
-    if (la.D)
-#pragma unroll
-      for (int k = 0; k < kLossPx; k += 4)
-        *reinterpret_cast<float4*>(la.D + (long long)b * FF + q0 + k) = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
-  }
-  const float* Ip = la.Ipart + (long long)b * a.G * FF;
+// Each thread takes kLossPx camera pixels of la.npos positions; pixel k of lane i of warp w is
+// 128 w + 32 k + i of the block's, so that every load, the four tap gathers among them, covers one run of
+// neighbouring pixels.  The taps, their weights and the remapped background of a thread's pixels serve
+// all its positions.  What bounds the pass is instructions (ncu, Poisson with background: 177-205 thread
+// instructions per pixel at two per cycle and SM, DRAM 12 % busy), hence the compile-time REMAP and ONE
+// (one intensity slice) and one reduction per position by one warp.
+// The loss terms of a block are summed as double-floats: per thread, then, for each position, by one warp
+// over the block's threads in a fixed order into one partial per (call entry, block); the sigma- and
+// z-gradient terms per thread, by a warp tree and in FP64 over the eight warps.
+// grid (F*F/(kLossThreads*kLossPx), ceil(nb / la.npos))
+struct LossShared {
+  float2 sum[kLossPosMax][kLossThreads];              // loss terms (hi, lo) of each thread
+  float red[kLossPosMax][4][kLossThreads / 32];       // sigma and z terms of each warp
+};
+
+template <int F, bool REMAP, bool ONE>
+__device__ __forceinline__ void loss_positions_body(const KArgs& a, const LossArgs& la, const uint3 bid, LossShared& sm) {
+  constexpr int FF = F * F, NB = loss_blocks<F>(), NW = kLossThreads / 32;
+  const int b0 = bid.y * la.npos, nb = min(la.npos, a.nb - b0);
+  const int q0 = bid.x * kLossThreads * kLossPx + (threadIdx.x >> 5) * 32 * kLossPx + (threadIdx.x & 31);
+  const int G = ONE ? 1 : la.Gsum;
+  const bool need = la.D || la.loss_part;
   int tb[kLossPx];
   float2 tw[kLossPx];
-  if (la.remap) {
-#pragma unroll
-    for (int k = 0; k < kLossPx; k += 4) {
-      const int4 t4 = *reinterpret_cast<const int4*>(la.tap_base + q0 + k);
-      const float4 w01 = *reinterpret_cast<const float4*>(la.tap_w + q0 + k);
-      const float4 w23 = *reinterpret_cast<const float4*>(la.tap_w + q0 + k + 2);
-      tb[k] = t4.x; tb[k + 1] = t4.y; tb[k + 2] = t4.z; tb[k + 3] = t4.w;
-      tw[k] = make_float2(w01.x, w01.y); tw[k + 1] = make_float2(w01.z, w01.w);
-      tw[k + 2] = make_float2(w23.x, w23.y); tw[k + 3] = make_float2(w23.z, w23.w);
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < kLossPx; ++k) { tb[k] = 0; tw[k] = make_float2(0.f, 0.f); }
-  }
-  float d[kLossPx];
-  float th = 0.f, tl = 0.f, sh = 0.f, sl = 0.f;   // double-float sums of the loss and sigma terms
-  float zh = 0.f, zl = 0.f;                       // and of the z terms
+  float Ib[kLossPx];                                  // background at the camera pixels
 #pragma unroll
   for (int k = 0; k < kLossPx; ++k) {
-    const int q = q0 + k;
-    float Is, Ib, srow, scol;
-    bool valid;
-    predict_pixel<F>(la, Ip, la.Gsum, q, tb[k], tw[k], Is, Ib, valid, srow, scol);
-    const float Ic = Is + Ib;
-    if (la.I_pred) la.I_pred[(long long)j * FF + q] = valid ? Ic : 0.f;
-    d[k] = 0.f;
-    if (la.D || la.loss_part) {
-      bool use = valid;
-      if (la.mask) use = use && (la.mask[(la.mask_per_frame ? (long long)j * FF : 0) + q] != 0);
-      if (use) {
-        float Ih = __ldg(la.Imeas + (long long)j * FF + q);
-        float Ie = Ic + la.eps;
-        if (la.loss_kind == 2) {                       // shifted Poisson
+    const int q = q0 + 32 * k;
+    tb[k] = q;
+    tw[k] = make_float2(0.f, 0.f);
+    Ib[k] = 0.f;
+    if (REMAP) {
+      tb[k] = __ldg(la.tap_base + q);
+      tw[k] = __ldg(la.tap_w + q);
+      if (la.bg && tb[k] >= 0)
+        Ib[k] = bilinear(tw[k], __ldg(la.bg + tb[k]), __ldg(la.bg + tb[k] + 1), __ldg(la.bg + tb[k] + F),
+                         __ldg(la.bg + tb[k] + F + 1));
+    } else if (la.bg) {
+      Ib[k] = __ldg(la.bg + q);
+    }
+  }
+  const float* Ip = la.Ipart + (long long)b0 * a.G * FF;
+  for (int n = 0; n < nb; ++n, Ip += (long long)a.G * FF) {
+    const int j = batch_pos(a, a.batch_off + b0 + n); // uniform over the block
+    float th = 0.f, tl = 0.f, sh = 0.f, sl = 0.f;     // double-float sums of the loss and sigma terms
+    float zh = 0.f, zl = 0.f;                         // and of the z terms
+    const long long frame = (long long)max(j, 0) * FF + q0;
+    float Is[kLossPx], Im[kLossPx], d[kLossPx];
+    bool use[kLossPx];
+#pragma unroll
+    for (int k = 0; k < kLossPx; ++k) {               // all loads first
+      Is[k] = Im[k] = d[k] = 0.f;
+      use[k] = j >= 0 && (!REMAP || tb[k] >= 0);      // outside the remap's grid: 0, and not in the loss
+      if (use[k]) {
+        if (REMAP)
+          Is[k] = bilinear(tw[k], model_I(Ip, G, FF, tb[k]), model_I(Ip, G, FF, tb[k] + 1),
+                           model_I(Ip, G, FF, tb[k] + F), model_I(Ip, G, FF, tb[k] + F + 1));
+        else
+          Is[k] = model_I(Ip, G, FF, tb[k]);
+      }
+      if (need) Im[k] = __ldg(la.Imeas + frame + 32 * k);
+    }
+    if (la.I_pred && j >= 0) {
+#pragma unroll
+      for (int k = 0; k < kLossPx; ++k) la.I_pred[frame + 32 * k] = Is[k] + Ib[k];
+    }
+    if (!need) continue;
+    if (la.mask) {
+      const uint8_t* m = la.mask + (la.mask_per_frame ? frame : (long long)q0);
+#pragma unroll
+      for (int k = 0; k < kLossPx; ++k) use[k] = use[k] && m[32 * k] != 0;
+    }
+    if (la.loss_kind == 0) {
+#pragma unroll
+      for (int k = 0; k < kLossPx; ++k) {
+        if (!use[k]) continue;
+        const float se = sqrtf(Is[k] + Ib[k] + la.eps), diff = se - sqrtf(Im[k]);
+        df_add(th, tl, diff * diff);
+        d[k] = __fdividef(diff, se);                  // 2 ulp: ample for a gradient
+      }
+    } else {
+      const bool shifted = la.loss_kind == 2;         // shifted Poisson
+#pragma unroll
+      for (int k = 0; k < kLossPx; ++k) {
+        if (!use[k]) continue;
+        float Ie = Is[k] + Ib[k] + la.eps, Ih = Im[k];
+        if (shifted) {
           Ie += la.read_var;
           Ih = fmaxf(Ih + la.read_var, 0.f);
         }
-        if (la.loss_kind == 0) {
-          const float se = sqrtf(Ie), diff = se - sqrtf(Ih);
-          df_add(th, tl, diff * diff);
-          d[k] = __fdividef(diff, se);                 // 2 ulp: ample for a gradient
-        } else {
-          df_add(th, tl, poisson_term(Ie, Ih));
-          d[k] = __fdividef(Ie - Ih, Ie);
-        }
-      }
-      if (la.sig_part) df_add(sh, sl, d[k] * Is);
-      if (la.z_part && d[k] != 0.f) {
-        const float2 rz = __ldg(la.tap_dz + q);
-        df_add(zh, zl, d[k] * fmaf(srow, rz.x, scol * rz.y));
+        df_add(th, tl, poisson_term(Ie, Ih));
+        d[k] = __fdividef(Ie - Ih, Ie);
       }
     }
-  }
-  if (la.D)
+    if (la.D) {
+      float* Dq = la.D + (long long)(b0 + n) * FF + q0;
 #pragma unroll
-    for (int k = 0; k < kLossPx; k += 4)
-      *reinterpret_cast<float4*>(la.D + (long long)b * FF + q0 + k) = make_float4(d[k], d[k + 1], d[k + 2], d[k + 3]);
-  if (!la.loss_part && !la.sig_part && !la.z_part) return;
-  if (la.loss_part) df_warp_sum(th, tl);           // each sum only when its output is requested
-  if (la.sig_part) df_warp_sum(sh, sl);            // (uniform branches)
-  if (la.z_part) df_warp_sum(zh, zl);
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = th;
-    red[1][threadIdx.x >> 5] = tl;
-    red[2][threadIdx.x >> 5] = sh;
-    red[3][threadIdx.x >> 5] = sl;
-    red[4][threadIdx.x >> 5] = zh;
-    red[5][threadIdx.x >> 5] = zl;
+      for (int k = 0; k < kLossPx; ++k) Dq[32 * k] = d[k];
+    }
+    if (la.loss_part) sm.sum[n][threadIdx.x] = make_float2(th, tl);
+    if (la.sig_part) {
+#pragma unroll
+      for (int k = 0; k < kLossPx; ++k) df_add(sh, sl, d[k] * Is[k]);
+      df_warp_sum(sh, sl);
+    }
+    if (REMAP && la.z_part) {                         // slopes of the interpolant of field + background
+#pragma unroll
+      for (int k = 0; k < kLossPx; ++k) {
+        if (d[k] == 0.f) continue;
+        const int u = tb[k];
+        const float2 w = tw[k];
+        float i00 = model_I(Ip, G, FF, u), i01 = model_I(Ip, G, FF, u + 1);
+        float i10 = model_I(Ip, G, FF, u + F), i11 = model_I(Ip, G, FF, u + F + 1);
+        if (la.bg) {
+          i00 += __ldg(la.bg + u); i01 += __ldg(la.bg + u + 1);
+          i10 += __ldg(la.bg + u + F); i11 += __ldg(la.bg + u + F + 1);
+        }
+        const float srow = ((1.f - w.y) * i10 + w.y * i11) - ((1.f - w.y) * i00 + w.y * i01);
+        const float scol = (1.f - w.x) * (i01 - i00) + w.x * (i11 - i10);
+        const float2 rz = __ldg(la.tap_dz + q0 + 32 * k);
+        df_add(zh, zl, d[k] * fmaf(srow, rz.x, scol * rz.y));
+      }
+      df_warp_sum(zh, zl);
+    }
+    if ((la.sig_part || la.z_part) && (threadIdx.x & 31) == 0) {
+      const int wi = threadIdx.x >> 5;
+      sm.red[n][0][wi] = sh;
+      sm.red[n][1][wi] = sl;
+      sm.red[n][2][wi] = zh;
+      sm.red[n][3][wi] = zl;
+    }
   }
+  if (!la.loss_part && !la.sig_part && !la.z_part) return;
   __syncthreads();
-  if (threadIdx.x < 3) {
-    double sum = 0.0;
-    for (int wi = 0; wi < kLossThreads / 32; ++wi)
-      sum += (double)red[2 * threadIdx.x][wi] + (double)red[2 * threadIdx.x + 1][wi];
-    double* out = threadIdx.x == 0 ? la.loss_part : (threadIdx.x == 1 ? la.sig_part : la.z_part);
-    if (out) out[(long long)i * NB + bid.x] = sum;
+  const long long part = (long long)(a.batch_off + b0) * NB + bid.x;
+  if (la.loss_part) {
+    static_assert(kLossPosMax <= NW, "one warp per position");
+    const int n = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (n < nb) {
+      float2 v = sm.sum[n][lane];
+#pragma unroll
+      for (int i = 1; i < NW; ++i) {
+        const float2 u = sm.sum[n][lane + 32 * i];
+        df_add_df(v.x, v.y, u.x, u.y);
+      }
+      df_warp_sum(v.x, v.y);
+      if (lane == 0) la.loss_part[part + (long long)n * NB] = (double)v.x + (double)v.y;
+    }
+  }
+  if (la.sig_part || la.z_part) {
+    const int n = threadIdx.x >> 1, kind = threadIdx.x & 1;
+    double* out = kind == 0 ? la.sig_part : la.z_part;
+    if (n < nb && out) {
+      double sum = 0.0;
+      for (int wi = 0; wi < NW; ++wi) sum += (double)sm.red[n][2 * kind][wi] + (double)sm.red[n][2 * kind + 1][wi];
+      out[part + (long long)n * NB] = sum;
+    }
   }
 }
 
 template <int F>
-__global__ void __launch_bounds__(kLossThreads)
+__device__ __forceinline__ void loss_body(const KArgs& a, const LossArgs& la, const uint3 bid) {
+  __shared__ LossShared sm;
+  if (la.remap) {
+    if (la.Gsum == 1) loss_positions_body<F, true, true>(a, la, bid, sm);
+    else loss_positions_body<F, true, false>(a, la, bid, sm);
+  } else {
+    if (la.Gsum == 1) loss_positions_body<F, false, true>(a, la, bid, sm);
+    else loss_positions_body<F, false, false>(a, la, bid, sm);
+  }
+}
+
+template <int F>
+__global__ void __launch_bounds__(kLossThreads, 4)
 k_loss(KArgs a, LossArgs la) {
   pdl_wait();
   pdl_trigger();

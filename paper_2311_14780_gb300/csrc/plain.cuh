@@ -187,7 +187,8 @@ int plain_adjoint(ptycho_plan& p, const CallArgs& c, float2* psi, float* Ibuf, f
     PTY_LAUNCH(p, kRowFwd, st, k_pl_rows<F, false><<<dim3(F / RowCfg<F>::RPB, frames), RowCfg<F>::threads, RowCfg<F>::smem, st>>>(psi, p.d_tw));
     PTY_LAUNCH(p, kColFwd, st, k_pl_cols<F, false><<<dim3(F / ColCfg<F>::W, frames), ColCfg<F>::threads, ColCfg<F>::smem_xch, st>>>(psi, p.d_tw, inv));
     PTY_LAUNCH(p, kColFwd, st, k_pl_intensity<F><<<dim3(FF / 256, a.nb), 256, 0, st>>>(psi, Ibuf, LM));
-    PTY_LAUNCH(p, kLoss, st, k_loss<F><<<dim3(loss_blocks<F>(), a.nb), kLossThreads, 0, st>>>(a, la));
+    la.npos = loss_positions(F, a.nb, p.sms);
+    PTY_LAUNCH(p, kLoss, st, k_loss<F><<<dim3(loss_blocks<F>(), (a.nb + la.npos - 1) / la.npos), kLossThreads, 0, st>>>(a, la));
     if (p.remap) PTY_LAUNCH(p, kRemapAdj, st, k_remap_adj<F><<<dim3(FF / 256, (a.nb + kRtPos - 1) / kRtPos), 256, 0, st>>>(a, aa));
     PTY_LAUNCH(p, kColAdj, st, k_pl_mul<F><<<dim3(FF / 256, LM, a.nb), 256, 0, st>>>(psi, p.remap ? Gbuf : Dbuf, LM));
     PTY_LAUNCH(p, kColAdj, st, k_pl_cols<F, true><<<dim3(F / ColCfg<F>::W, frames), ColCfg<F>::threads, ColCfg<F>::smem_xch, st>>>(psi, p.d_tw, inv));

@@ -193,6 +193,7 @@ void fill_round(Site* s, int r, ptycho::SiteRound& w, int& tiles, int* counts, p
   la.loss_part = p.d_loss_part;
   la.remap = p.remap;
   la.Gsum = p.G;
+  la.npos = ptycho::loss_positions(F, a.nb, p.sms);
   la.tap_dz = p.d_tap_dz;
   AdjArgs aa{};
   aa.D = p.d_D;
@@ -231,7 +232,7 @@ void fill_round(Site* s, int r, ptycho::SiteRound& w, int& tiles, int* counts, p
   }
   counts[kMpRowFwd] = (F / rows) * p.L * a.nb;
   counts[kMpColFwd] = (F / cols) * p.G * a.nb;
-  counts[kMpLoss] = (F * F / (kLossThreads * kLossPx)) * a.nb;
+  counts[kMpLoss] = (F * F / (kLossThreads * kLossPx)) * ((a.nb + la.npos - 1) / la.npos);
   counts[kMpRemapAdj] = p.remap ? (F * F / 256) * ((a.nb + kRtPos - 1) / kRtPos) : 0;
   counts[kMpColAdj] = counts[kMpColFwd];
   counts[kMpRowAdj] = fused ? 0 : (F / (256 / (T * kAdjSlots))) * LM;

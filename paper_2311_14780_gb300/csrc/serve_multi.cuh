@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_multi(RoundTab rt) {
   const int loc = load_site(rt, kMpLoss, w);
   pdl_wait();
   pdl_trigger();
-  loss_body<F>(w.a, w.la, unflatten(loc, loss_blocks<F>(), w.a.nb));
+  loss_body<F>(w.a, w.la, unflatten(loc, loss_blocks<F>(), w.a.nb));   // y: the group of w.la.npos positions
 }
 
 template <int F>
