@@ -505,7 +505,12 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
       if (obj_atomic) continue;
       if (nsets > 1 && k > 0 && cudaStreamWaitEvent(cs, p.ev_og[(k - 1) % nsets], 0) != cudaSuccess)
         return PTYCHO_ECUDA;
-      PTY_LAUNCH(p, kObjGrad, cs, launch_pdl(k_obj_grad<F>, dim3(max_tiles, p.L), 256, 0, cs, S, c.gO, a));
+      // with one mode the slot is the sum over the modes: the listing kernel adds the same values in the
+      // same order (400 positions of 512^2: 335 -> 156 us, the other walks every position of the batch)
+      if (p.M == 1 && p.nchunks == 1)
+        PTY_LAUNCH(p, kObjGrad, cs, launch_pdl(k_obj_grad_l<F, false, 4>, dim3(max_tiles, p.L), 256, 0, cs, S, c.gO, a));
+      else
+        PTY_LAUNCH(p, kObjGrad, cs, launch_pdl(k_obj_grad<F>, dim3(max_tiles, p.L), 256, 0, cs, S, c.gO, a));
       if (nsets > 1 && cudaEventRecord(p.ev_og[k % nsets], cs) != cudaSuccess) return PTYCHO_ECUDA;
     }
   }
