@@ -51,6 +51,11 @@ extern "C" {
 #define PTYCHO_EBUSY (-8)        /* serving: no free slot, or the HBM budget is exhausted  */
 
 /* Pipeline variants (ptycho_geom_t.flags).  All give the same results up to FP32 rounding.
+ * Without a flag (or with NO_PDL alone) a plan that keeps all modes of a position in the scratch, with
+ * at least two positions per batch and two fields per position (one at F <= 128), transforms pairs of
+ * positions in the packed FP32 lanes (csrc/pair.cuh), where its row adjoint's block fits (any
+ * count up to 10 modes; up to 20, 40 and 72 at F = 256, 128 and 64 where the count fills whole warps in
+ * a block of at most 320 threads).  Any other flag selects the one-field passes, whose variants and defaults the following describes.
  * RECOMPUTE_COLUMNS: the adjoint recomputes the column DFT from the kept row-pass output
  *   instead of keeping Psi (less memory traffic, one more 1D pass per evaluation); the
  *   default for F >= 256, where it measured faster.

@@ -1701,11 +1701,16 @@ __global__ void k_sigma_grad(const int32_t* __restrict__ bidx, int nbatch, int J
                              int nblk, const float* __restrict__ sigma, float* __restrict__ g);
 __global__ void k_sum_sets(const float* __restrict__ acc, int nsets, long long n, float* __restrict__ out);
 __global__ void k_tick(int* t);
-__global__ void k_adam_dev(float* __restrict__ theta, const float* __restrict__ grad, float* __restrict__ m,
-                           float* __restrict__ v, long long n, float lr, float b1, float b2, float eps,
-                           const int* __restrict__ t_dev);
-__global__ void k_adam(float* __restrict__ theta, const float* __restrict__ grad, float* __restrict__ m,
-                       float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
-                       float c2);
+// Real parameters of one array with their gradient, moments and learning rate.
+struct AdamArray {
+  float* theta;
+  const float* grad;
+  float* m;
+  float* v;
+  long long n;
+  float lr;
+};
+__global__ void k_adam_dev(AdamArray p, AdamArray q, float b1, float b2, float eps, const int* __restrict__ t_dev);
+__global__ void k_adam(AdamArray p, AdamArray q, float b1, float b2, float eps, float c1, float c2);
 
 }  // namespace ptycho

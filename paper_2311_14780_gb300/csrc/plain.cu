@@ -59,10 +59,11 @@ extern "C" int ptycho_plain_step(ptycho_plan_t* p, ptycho_adam_t* s, float* O, f
   const double c1 = 1.0 / (1.0 - pow((double)s->beta1, (double)s->t));
   const double c2 = 1.0 / (1.0 - pow((double)s->beta2, (double)s->t));
   const int grid = 4 * p->sms;
-  ptycho::k_adam<<<grid, 256, 0, st>>>(O, reinterpret_cast<const float*>(p->d_gO), s->mO, s->vO, 2 * p->O_numel,
-                                       s->lr_O, s->beta1, s->beta2, s->eps, (float)c1, (float)c2);
-  ptycho::k_adam<<<grid, 256, 0, st>>>(P, reinterpret_cast<const float*>(p->d_gP), s->mP, s->vP, 2 * p->P_numel,
-                                       s->lr_P, s->beta1, s->beta2, s->eps, (float)c1, (float)c2);
+  const ptycho::AdamArray none{};
+  const ptycho::AdamArray aO{O, reinterpret_cast<const float*>(p->d_gO), s->mO, s->vO, 2 * p->O_numel, s->lr_O};
+  const ptycho::AdamArray aP{P, reinterpret_cast<const float*>(p->d_gP), s->mP, s->vP, 2 * p->P_numel, s->lr_P};
+  ptycho::k_adam<<<grid, 256, 0, st>>>(aO, none, s->beta1, s->beta2, s->eps, (float)c1, (float)c2);
+  ptycho::k_adam<<<grid, 256, 0, st>>>(aP, none, s->beta1, s->beta2, s->eps, (float)c1, (float)c2);
   p->last_launches += 2;
   return cudaGetLastError() == cudaSuccess ? PTYCHO_OK : PTYCHO_ECUDA;
 }

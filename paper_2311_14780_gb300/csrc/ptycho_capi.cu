@@ -113,16 +113,21 @@ k_sum_sets(const float* __restrict__ acc, int nsets, long long n, float* __restr
 }
 
 // Adam (Kingma & Ba) on real parameters; c1, c2 are the bias corrections 1/(1-beta^t).
+__device__ __forceinline__ void adam_element(const AdamArray& p, long long i, float b1, float b2, float eps, float c1, float c2) {
+  const float g = p.grad[i];
+  const float mi = fmaf(b1, p.m[i], (1.f - b1) * g);
+  const float vi = fmaf(b2, p.v[i], (1.f - b2) * g * g);
+  p.m[i] = mi;
+  p.v[i] = vi;
+  p.theta[i] -= p.lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+}
+// Objects and probes in one launch (q is the second array, n = 0 for none): 28 bytes per parameter bound it on
+// large plans, the launch itself on small ones.
 __global__ void __launch_bounds__(256)
-k_adam(float* __restrict__ theta, const float* __restrict__ grad, float* __restrict__ m, float* __restrict__ v,
-       long long n, float lr, float b1, float b2, float eps, float c1, float c2) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float g = grad[i];
-    const float mi = fmaf(b1, m[i], (1.f - b1) * g);
-    const float vi = fmaf(b2, v[i], (1.f - b2) * g * g);
-    m[i] = mi;
-    v[i] = vi;
-    theta[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+k_adam(AdamArray p, AdamArray q, float b1, float b2, float eps, float c1, float c2) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.n + q.n; i += (long long)gridDim.x * blockDim.x) {
+    if (i < p.n) adam_element(p, i, b1, b2, eps, c1, c2);
+    else adam_element(q, i - p.n, b1, b2, eps, c1, c2);
   }
 }
 
@@ -133,21 +138,15 @@ __global__ void k_tick(int* t) {
 
 // Adam with the step counter read on the device (for graph replays).
 __global__ void __launch_bounds__(256)
-k_adam_dev(float* __restrict__ theta, const float* __restrict__ grad, float* __restrict__ m, float* __restrict__ v,
-           long long n, float lr, float b1, float b2, float eps, const int* __restrict__ t_dev) {
+k_adam_dev(AdamArray p, AdamArray q, float b1, float b2, float eps, const int* __restrict__ t_dev) {
   const float t = (float)(*t_dev);
   const float c1 = 1.0f / (1.0f - powf(b1, t));
   const float c2 = 1.0f / (1.0f - powf(b2, t));
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float g = grad[i];
-    const float mi = fmaf(b1, m[i], (1.f - b1) * g);
-    const float vi = fmaf(b2, v[i], (1.f - b2) * g * g);
-    m[i] = mi;
-    v[i] = vi;
-    theta[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.n + q.n; i += (long long)gridDim.x * blockDim.x) {
+    if (i < p.n) adam_element(p, i, b1, b2, eps, c1, c2);
+    else adam_element(q, i - p.n, b1, b2, eps, c1, c2);
   }
 }
-
 
 long long prof_begin(ptycho_plan& p, int kind, cudaStream_t st) {
   if (!p.prof) return -1;
@@ -170,6 +169,7 @@ void prof_end(ptycho_plan& p, long long idx, cudaStream_t st) {
 
 }  // namespace ptycho
 
+using ptycho::AdamArray;
 using ptycho::CallArgs;
 using ptycho::CallKind;
 
@@ -623,7 +623,9 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
     if (g->M == 1 || (rpb * z.T * g->M <= ptycho::kRowAdjPairThreads && pair_sizes(F, g->M, rpb).smem <= ptycho::kRowAdjLSmemMax)) {
       p->pair = 1;
       p->rpb_pair = rpb;
-      if ((p->B & 1) && p->B < g->J) p->B += g->scratch_bytes > 0 || p->B == ptycho::kMaxB ? -1 : 1;
+      // whole pairs of positions, within the budget
+      if ((p->B & 1) && (p->B < g->J || (p->B + 1) * LM * FF8 > p->scratch_budget))
+        p->B += g->scratch_bytes > 0 || p->B == ptycho::kMaxB || (p->B + 1) * LM * FF8 > p->scratch_budget ? -1 : 1;
     }
   }
   int colblocks = 0;
@@ -1077,67 +1079,37 @@ int ptycho_step(ptycho_plan_t* p, ptycho_adam_t* s, float* O, float* P, float* s
   const long long FF = (long long)p->F * p->F;
   const long long nD = 2ll * p->L * p->J;
   const int grid = 4 * p->sms;
+  const AdamArray none{};
+  const AdamArray aO{O, reinterpret_cast<const float*>(p->d_gO), s->mO, s->vO, nO, s->lr_O};
+  const AdamArray aP{P, reinterpret_cast<const float*>(p->d_gP), s->mP, s->vP, nP, s->lr_P};
+  const AdamArray aS{sigma, p->d_gsig, s->m_sigma, s->v_sigma, p->J, s->lr_sigma};
+  const AdamArray aB{bg, p->d_gbg, s->m_bg, s->v_bg, FF, s->lr_bg};
+  const AdamArray aD{p->d_delta, p->d_gdelta, s->m_delta, s->v_delta, nD, s->lr_delta};
+  float c1 = 0.f, c2 = 0.f;
   if (s->t_dev) {
     // device step counter: the update can be captured once and replayed
     ptycho::k_tick<<<1, 32, 0, st>>>(s->t_dev);
     ++p->last_launches;
     if (cudaGetLastError() != cudaSuccess) return PTYCHO_ECUDA;
-    long long ev = ptycho::prof_begin(*p, ptycho::kAdam, st);
-    ptycho::k_adam_dev<<<grid, 256, 0, st>>>(O, reinterpret_cast<const float*>(p->d_gO), s->mO, s->vO, nO, s->lr_O,
-                                             s->beta1, s->beta2, s->eps, s->t_dev);
-    ptycho::k_adam_dev<<<grid, 256, 0, st>>>(P, reinterpret_cast<const float*>(p->d_gP), s->mP, s->vP, nP, s->lr_P,
-                                             s->beta1, s->beta2, s->eps, s->t_dev);
-    p->last_launches += 2;
-    if (opt_sigma) {
-      ptycho::k_adam_dev<<<(p->J + 255) / 256, 256, 0, st>>>(sigma, p->d_gsig, s->m_sigma, s->v_sigma, p->J,
-                                                             s->lr_sigma, s->beta1, s->beta2, s->eps, s->t_dev);
-      ++p->last_launches;
-    }
-    if (opt_bg) {
-      ptycho::k_adam_dev<<<(int)((FF + 255) / 256), 256, 0, st>>>(bg, p->d_gbg, s->m_bg, s->v_bg, FF, s->lr_bg,
-                                                                   s->beta1, s->beta2, s->eps, s->t_dev);
-      ++p->last_launches;
-    }
-    if (opt_delta) {
-      ptycho::k_adam_dev<<<(int)((nD + 255) / 256), 256, 0, st>>>(p->d_delta, p->d_gdelta, s->m_delta, s->v_delta, nD,
-                                                                   s->lr_delta, s->beta1, s->beta2, s->eps, s->t_dev);
-      ++p->last_launches;
-    }
-    if (cudaGetLastError() != cudaSuccess) return PTYCHO_ECUDA;
-    ptycho::prof_end(*p, ev, st);
-    return PTYCHO_OK;
+  } else {
+    s->t += 1;
+    c1 = (float)(1.0 / (1.0 - pow((double)s->beta1, (double)s->t)));
+    c2 = (float)(1.0 / (1.0 - pow((double)s->beta2, (double)s->t)));
   }
-  s->t += 1;
-  const double c1 = 1.0 / (1.0 - pow((double)s->beta1, (double)s->t));
-  const double c2 = 1.0 / (1.0 - pow((double)s->beta2, (double)s->t));
-  long long ev = ptycho::prof_begin(*p, ptycho::kAdam, st);
-  ptycho::k_adam<<<grid, 256, 0, st>>>(O, reinterpret_cast<const float*>(p->d_gO), s->mO, s->vO, nO, s->lr_O,
-                                       s->beta1, s->beta2, s->eps, (float)c1, (float)c2);
-  ++p->last_launches;
+  auto launch = [&](int blocks, const AdamArray& x, const AdamArray& y) {
+    if (s->t_dev)
+      ptycho::k_adam_dev<<<blocks, 256, 0, st>>>(x, y, s->beta1, s->beta2, s->eps, s->t_dev);
+    else
+      ptycho::k_adam<<<blocks, 256, 0, st>>>(x, y, s->beta1, s->beta2, s->eps, c1, c2);
+    ++p->last_launches;
+  };
+  const long long ev = ptycho::prof_begin(*p, ptycho::kAdam, st);
+  launch(grid, aO, aP);
   if (cudaGetLastError() != cudaSuccess) return PTYCHO_ECUDA;
   ptycho::prof_end(*p, ev, st);
-  ev = ptycho::prof_begin(*p, ptycho::kAdam, st);
-  ptycho::k_adam<<<grid, 256, 0, st>>>(P, reinterpret_cast<const float*>(p->d_gP), s->mP, s->vP, nP, s->lr_P,
-                                       s->beta1, s->beta2, s->eps, (float)c1, (float)c2);
-  ++p->last_launches;
-  if (cudaGetLastError() != cudaSuccess) return PTYCHO_ECUDA;
-  ptycho::prof_end(*p, ev, st);
-  if (opt_sigma) {
-    ptycho::k_adam<<<(p->J + 255) / 256, 256, 0, st>>>(sigma, p->d_gsig, s->m_sigma, s->v_sigma, p->J, s->lr_sigma,
-                                                       s->beta1, s->beta2, s->eps, (float)c1, (float)c2);
-    ++p->last_launches;
-  }
-  if (opt_bg) {
-    ptycho::k_adam<<<(int)((FF + 255) / 256), 256, 0, st>>>(bg, p->d_gbg, s->m_bg, s->v_bg, FF, s->lr_bg, s->beta1,
-                                                             s->beta2, s->eps, (float)c1, (float)c2);
-    ++p->last_launches;
-  }
-  if (opt_delta) {
-    ptycho::k_adam<<<(int)((nD + 255) / 256), 256, 0, st>>>(p->d_delta, p->d_gdelta, s->m_delta, s->v_delta, nD,
-                                                             s->lr_delta, s->beta1, s->beta2, s->eps, (float)c1,
-                                                             (float)c2);
-    ++p->last_launches;
-  }
+  if (opt_sigma) launch((p->J + 255) / 256, aS, none);
+  if (opt_bg) launch((int)((FF + 255) / 256), aB, none);
+  if (opt_delta) launch((int)((nD + 255) / 256), aD, none);
   if (cudaGetLastError() != cudaSuccess) return PTYCHO_ECUDA;
   return PTYCHO_OK;
 }

@@ -454,12 +454,9 @@ int enqueue_iteration(Site* s, cudaStream_t st) {
   float* vO = mO + nO;
   float* mP = vO + nO;
   float* vP = mP + nP;
-  const int grid = 4 * p->sms;
-  ptycho::k_adam_dev<<<grid, 256, 0, st>>>(s->data.O, reinterpret_cast<const float*>(p->d_gO), mO, vO, nO,
-                                           s->data.lr_O, s->data.beta1, s->data.beta2, s->data.eps, s->t_dev);
-  if (cudaGetLastError() != cudaSuccess) return PTYCHO_ECUDA;
-  ptycho::k_adam_dev<<<grid, 256, 0, st>>>(s->data.P, reinterpret_cast<const float*>(p->d_gP), mP, vP, nP,
-                                           s->data.lr_P, s->data.beta1, s->data.beta2, s->data.eps, s->t_dev);
+  const ptycho::AdamArray aO{s->data.O, reinterpret_cast<const float*>(p->d_gO), mO, vO, nO, s->data.lr_O};
+  const ptycho::AdamArray aP{s->data.P, reinterpret_cast<const float*>(p->d_gP), mP, vP, nP, s->data.lr_P};
+  ptycho::k_adam_dev<<<4 * p->sms, 256, 0, st>>>(aO, aP, s->data.beta1, s->data.beta2, s->data.eps, s->t_dev);
   if (cudaGetLastError() != cudaSuccess) return PTYCHO_ECUDA;
   return PTYCHO_OK;
 }
