@@ -125,11 +125,10 @@ int prepare_kernels() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_adj_p<F, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowAdjLSmemMax);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_adj_p<F, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowAdjLSmemMax);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_adj_p1<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, row_adj_p1_smem<F>());
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_rows<F, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowCfg<F>::smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_rows<F, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowCfg<F>::smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_rows<F, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowCfg<F>::smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_cols<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColCfg<F>::smem_xch);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_cols<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColCfg<F>::smem_xch);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_cols<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, shift_cols_smem<F>());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_rows<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, shift_rows_smem<F>());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_rows_adj<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, shift_rows_smem<F>());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_shift_cols_adj<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, shift_cols_smem<F>());
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_czt_row_fwd<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, CztRowCfg<F>::smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_czt_col_fwd<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, CztColCfg<F>::smem_fwd);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_czt_col_adj<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, CztColCfg<F>::smem_adj);
@@ -274,20 +273,20 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
     // forward: all chunks accumulate the model intensity
     // fractional offsets: shift the batch's object windows into the patch buffer
     const long long set_P = (long long)p.B * p.L * FF;
+    const dim3 srow_grid(F / RowCfg<F>::RPB, p.L, a.nb), scol_grid(F / ColCfg<F>::W, p.L, a.nb);
     ShiftArgs sh{};
     if (shifted) {
       sh.delta = p.d_delta;
-      sh.T = p.d_shT + set * set_P;
-      sh.Q = p.d_shQ + set * set_P;
-      float2* Pt = p.d_shP + set * set_P;
-      const dim3 rgrid(F / RowCfg<F>::RPB, p.L, a.nb), cgrid(F / ColCfg<F>::W, p.L, a.nb);
-      sh.dst = sh.T; sh.dst_b = (long long)p.L * FF; sh.dst_l = FF; sh.scale = 1.0f;
-      PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_rows<F, false, true>, rgrid, row_blk, RowCfg<F>::smem, cs, c.O, a, sh));
-      PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_cols<F, false>, cgrid, col_blk, ColCfg<F>::smem_xch, cs, a, sh));
-      sh.src = sh.T; sh.src_b = (long long)p.L * FF; sh.src_l = FF;
-      sh.dst = Pt; sh.scale = 1.0f / (float)FF;
-      PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_rows<F, true, false>, rgrid, row_blk, RowCfg<F>::smem, cs, c.O, a, sh));
-      a.patch = Pt;
+      sh.u = p.d_shT + set * set_P;
+      sh.g1 = p.d_shQ + set * set_P;
+      sh.patch = p.d_shP + set * set_P;
+      sh.slot = S;
+      sh.slot_b = (long long)p.C * FF;
+      sh.slot_l = (long long)p.M * FF;
+      sh.slot_pair = pair;
+      PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_cols<F>, scol_grid, col_blk, shift_cols_smem<F>(), cs, c.O, a, sh));
+      PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_rows<F>, srow_grid, row_blk, shift_rows_smem<F>(), cs, a, sh));
+      a.patch = sh.patch;
     }
     if constexpr (ResSupported<F>::value) {
       if (res) {                                      // all modes of the batch, frames on chip
@@ -473,16 +472,9 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
                                 p.rpb_adj, nsplit));
         if (nsets > 1 && cudaEventRecord(p.ev_radj[k % nsets], cs) != cudaSuccess) return PTYCHO_ECUDA;
         if (shifted) {                                // adjoint shift of the mode-summed patch gradients
-          const dim3 rgrid(F / RowCfg<F>::RPB, p.L, a.nb), cgrid(F / ColCfg<F>::W, p.L, a.nb);
-          sh.src = S; sh.src_b = (long long)p.C * FF; sh.src_l = (long long)p.M * FF; sh.src_pair = pair;
-          sh.dst = sh.T; sh.dst_b = (long long)p.L * FF; sh.dst_l = FF; sh.scale = 1.0f;
-          PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_rows<F, false, false>, rgrid, row_blk, RowCfg<F>::smem, cs, c.O, a, sh));
           sh.dpart = c.g_delta ? p.d_dpart : nullptr;
-          PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_cols<F, true>, cgrid, col_blk, ColCfg<F>::smem_xch, cs, a, sh));
-          sh.src = sh.T; sh.src_b = (long long)p.L * FF; sh.src_l = FF; sh.src_pair = 0;
-          sh.dst = S; sh.dst_b = (long long)p.C * FF; sh.dst_l = (long long)p.M * FF; sh.dst_pair = pair; sh.scale = 1.0f / (float)FF;
-          PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_rows<F, true, false>, rgrid, row_blk, RowCfg<F>::smem, cs, c.O, a, sh));
-          sh.dpart = nullptr;
+          PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_rows_adj<F>, srow_grid, row_blk, shift_rows_smem<F>(), cs, a, sh));
+          PTY_LAUNCH(p, kShift, cs, launch_pdl(k_shift_cols_adj<F>, scol_grid, col_blk, shift_cols_smem<F>(), cs, a, sh));
         }
         if (nsets > 1 && k > 0 && cudaStreamWaitEvent(cs, p.ev_og[(k - 1) % nsets], 0) != cudaSuccess)
           return PTYCHO_ECUDA;

@@ -95,8 +95,8 @@ struct ptycho_plan {
   float2* d_tap_dz = nullptr;                  // [F*F] d(row, col tap index)/dz
   double* d_z_part = nullptr;                  // [J][loss_blocks] z-gradient partials
   long long rt_cap = 0;                        // capacity of d_rt_idx / d_rt_w
-  float2* d_shT = nullptr;                     // [nsets][B][L][F][F] transform workspace
-  float2* d_shQ = nullptr;                     // [nsets][B][L][F][F] ramp * spectrum of the windows
+  float2* d_shT = nullptr;                     // [nsets][B][L][F][F] windows shifted along their columns
+  float2* d_shQ = nullptr;                     // [nsets][B][L][F][F] patch gradients after the row adjoint
   float2* d_shP = nullptr;                     // [nsets][B][L][F][F] shifted patches
   double* d_dpart = nullptr;                   // [J][L][F/W][2] position-gradient partials
   float* d_gdelta = nullptr;                   // [L][J][2] position gradient (ptycho_step)

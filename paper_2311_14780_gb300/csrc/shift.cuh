@@ -5,19 +5,25 @@
 // wavelength l is the F x F window at the integer position resampled at r + delta:
 //   p_delta = F2^-1[ ramp * F2 p ],   ramp(k) = exp(2 pi i (f(k_y) d_y + f(k_x) d_x)),
 // with f(k) = k/F for k < F/2 and (k - F)/F otherwise, the window taken as one period.
+// The ramp is a product of one factor per axis, so the shift is a shift of every column followed by one of
+// every row, each DFT, ramp, inverse DFT within one thread group: a pass per axis instead of the three
+// (rows, columns with the ramp, rows) of a 2D transform and back, and no spectrum kept for the adjoint.
 // Per position batch, before the forward row pass:
-//   k_shift_rows (window rows from O -> row DFT -> T)
-//   k_shift_cols (column DFT, * ramp, keep Q = ramp * DFT2(p) for the adjoint, inverse column DFT)
-//   k_shift_rows (inverse row DFT, / F^2 -> the batch's patch buffer, read by the row passes)
+//   k_shift_cols      (columns of the window, gathered from O) -> u
+//   k_shift_rows      (rows of u) -> the batch's patch buffer, read by the row passes
 // and after the adjoint row pass, on the mode-summed object-gradient patch g (the gradient
-// with respect to p_delta) in scratch slot (b, l*M):
-//   k_shift_rows (row DFT -> T)
-//   k_shift_cols (column DFT -> Ghat; position-gradient partials
-//                 dL/d delta_a = (1/F^2) Re sum_k conj(Ghat) (2 pi i f_a) Q, by Parseval's theorem;
-//                 * conj(ramp); inverse column DFT)
-//   k_shift_rows (inverse row DFT, / F^2 -> back into the slot: the adjoint-shifted patch
-//                 gradient that the object-gradient kernel adds into grad O)
-// All transforms are the unscaled two-stage register FFTs of fft_regs.cuh.
+// with respect to p_delta) in its scratch slot:
+//   k_shift_rows_adj  (rows: conjugate ramp) -> g'; with G, U the row spectra of g and u,
+//                     dL/d delta_x = -(2 pi / F) sum f_x Im(conj(G) ramp_x U)   (Parseval's theorem)
+//   k_shift_cols_adj  (columns: conjugate ramp) -> back into the slot: the adjoint-shifted patch gradient
+//                     that the object-gradient kernel adds into grad O; with G', U the column spectra of
+//                     g' and u, dL/d delta_y = -(2 pi / F) sum f_y Im(conj(G') U): u is
+//                     already shifted along its columns
+// A block's vectors share one ramp, evaluated once per block.  All transforms are the unscaled two-stage
+// register FFTs of fft_regs.cuh.
+// 400 positions of 256^2 x 4 modes x 3 wavelengths with every position optimised: 4.64 -> 4.46 ms per step
+// (112 -> 80 bytes of HBM traffic per window element, one ramp value per block and frequency instead of one
+// per element).
 #pragma once
 #include "kernels.cuh"
 
@@ -30,133 +36,198 @@ __device__ __forceinline__ float dft_freq(int k) {
 }
 
 struct ShiftArgs {
-  const float2* src;             // rows to transform (see k_shift_rows)
-  long long src_b, src_l;        // element strides of the source between positions and wavelengths
-  float2* dst;
-  long long dst_b, dst_l;
-  int src_pair, dst_pair;        // the source or destination is a slot of the pair passes: positions 2p and
-                                 // 2p+1 share rows of 2 F values (2p first)
-  float scale;                   // applied to the output (1 or 1/F^2)
   const float* delta;            // [L][J][2] fractional offsets (device)
-  float2* T;                     // [B][L][F][F] transform workspace of the batch
-  float2* Q;                     // [B][L][F][F] ramp * DFT2(window) of the batch
-  double* dpart;                 // [nbatch][L][F/W][2] position-gradient partials, or null
+  float2* u;                     // [B][L][F][F] windows shifted along their columns
+  float2* patch;                 // [B][L][F][F] shifted windows
+  float2* g1;                    // [B][L][F][F] patch gradients after the row adjoint
+  float2* slot;                  // patch gradients in the scratch: slot l*M of position b
+  long long slot_b, slot_l;      // its element strides between positions and wavelengths
+  int slot_pair;                 // a slot of the pair passes: positions 2p and 2p+1 share rows of 2 F
+                                 // values (2p first)
+  double* dpart;                 // [nbatch][L][F/W][2] position-gradient partials (y, x), or null
 };
 
-// Offset of row r of the patch of (position b, wavelength l).
-__device__ __forceinline__ long long patch_row(int b, int l, int r, int F, long long sb, long long sl, int pair) {
-  return pair ? 2 * ((b >> 1) * sb + l * sl + (long long)r * F) + (b & 1) * F : b * sb + l * sl + (long long)r * F;
+// Offset of row r of the patch of (position b, wavelength l) in the scratch, and between its rows.
+__device__ __forceinline__ long long slot_row(const ShiftArgs& sa, int b, int l, int r, int F) {
+  return sa.slot_pair ? 2 * ((b >> 1) * sa.slot_b + l * sa.slot_l + (long long)r * F) + (b & 1) * F
+                      : b * sa.slot_b + l * sa.slot_l + (long long)r * F;
 }
 
-// Row DFT of the F x F patches of the batch, one row per T threads.
-// INV = false: source rows in natural order -> forward DFT -> destination in natural order;
-// INV = true: the inverse.  FROM_O: the source rows are the object window at the integer
-// position (src/src_b/src_l unused).   grid (F/RPB, L, nb)
-template <int F, bool INV, bool FROM_O>
-__global__ void __launch_bounds__(RowCfg<F>::threads)
-k_shift_rows(const float2* __restrict__ O, KArgs a, ShiftArgs sa) {
-  pdl_wait();
-  pdl_trigger();
-  constexpr int N1 = FftShape<F>::N1, N2 = FftShape<F>::N2, T = RowCfg<F>::T;
-  extern __shared__ float2 smem[];
-  const int vec = threadIdx.x / T, t = threadIdx.x % T;
-  const int r = blockIdx.x * RowCfg<F>::RPB + vec;
-  const int l = blockIdx.y, b = blockIdx.z;
-  const int j = batch_pos(a, a.batch_off + b);
-  if (j < 0) return;                                  // uniform over the block
-  const float2* src = FROM_O ? O + a.obj_off[l] + (long long)(a.pos[(l * a.J + j) * 2] + r) * a.obj_w[l] +
-                                   a.pos[(l * a.J + j) * 2 + 1]
-                             : sa.src + patch_row(b, l, r, F, sa.src_b, sa.src_l, sa.src_pair);
-  float2* dst = sa.dst + patch_row(b, l, r, F, sa.dst_b, sa.dst_l, sa.dst_pair);
-  float2* xc = smem + vec * Xch<F>::region_rows;
-  float2 v[N2];
-  if (!INV) {
-#pragma unroll
-    for (int n2 = 0; n2 < N2; ++n2) v[n2] = src[t + N1 * n2];
-    fft_fwd_I2O<F>(v, t, xc, a.tw, WarpSync{});
-#pragma unroll
-    for (int sl = 0; sl < N2; ++sl) dst[idxO<F>(t, sl)] = cscale(v[sl], sa.scale);
-  } else {
-#pragma unroll
-    for (int sl = 0; sl < N2; ++sl) v[sl] = src[idxO<F>(t, sl)];
-    fft_inv_O2I<F>(v, t, xc, a.tw, WarpSync{});
-#pragma unroll
-    for (int n2 = 0; n2 < N2; ++n2) dst[t + N1 * n2] = cscale(v[n2], sa.scale);
+// exp(2 pi i f(k) d) for every k, by the whole block.
+template <int F>
+__device__ __forceinline__ void stage_ramp(float d, float2* ramp) {
+  for (int k = threadIdx.x; k < F; k += blockDim.x) {
+    float sn, cs;
+    sincospif(2.0f * dft_freq<F>(k) * d, &sn, &cs);
+    ramp[k] = make_float2(cs, sn);
   }
+  __syncthreads();
 }
 
-// Column pass of the shift on T (rows already transformed): column DFT, phase ramp
-// (ADJ: its conjugate, after the position-gradient partials), inverse column DFT, back to T.
-// Forward: Q <- ramp * spectrum.   grid (F/W, L, nb)
-template <int F, bool ADJ>
+// Sum over the block of double-float terms (256 threads), times ``scale``, in FP64; valid in thread 0.
+__device__ __forceinline__ double shift_block_sum(float hi, float lo, float (*red)[8], double scale) {
+  df_warp_sum(hi, lo);
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = hi;
+    red[1][threadIdx.x >> 5] = lo;
+  }
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < 8; ++w) s += (double)red[0][w] + (double)red[1][w];
+  return s * scale;
+}
+
+template <int F> __host__ __device__ constexpr int shift_cols_smem() { return ColCfg<F>::smem_xch + F * 8; }
+template <int F> __host__ __device__ constexpr int shift_rows_smem() { return RowCfg<F>::smem + F * 8; }
+
+// grid (F/W, L, nb)
+template <int F>
 __global__ void __launch_bounds__(ColCfg<F>::threads)
-k_shift_cols(KArgs a, ShiftArgs sa) {
+k_shift_cols(const float2* __restrict__ O, KArgs a, ShiftArgs sa) {
   pdl_wait();
   pdl_trigger();
   constexpr int N1 = FftShape<F>::N1, N2 = FftShape<F>::N2, W = ColCfg<F>::W;
   extern __shared__ float2 smem[];
-  __shared__ float red[4][ColCfg<F>::threads / 32];
+  float2* ramp = smem + W * Xch<F>::region_cols;
   const int c = threadIdx.x % W, t = threadIdx.x / W;
-  const int col = blockIdx.x * W + c;
-  const int l = blockIdx.y, b = blockIdx.z;
+  const int col = blockIdx.x * W + c, l = blockIdx.y, b = blockIdx.z;
   const int j = batch_pos(a, a.batch_off + b);
-  if (j < 0) {
-    if (ADJ && sa.dpart && threadIdx.x < 2)
-      sa.dpart[(((long long)(a.batch_off + b) * a.L + l) * gridDim.x + blockIdx.x) * 2 + threadIdx.x] = 0.0;
-    return;                                           // uniform over the block
-  }
-  const float dy = __ldg(sa.delta + (l * a.J + j) * 2), dx = __ldg(sa.delta + (l * a.J + j) * 2 + 1);
-  float2* base = sa.T + ((long long)b * a.L + l) * F * F + col;
-  float2* qb = sa.Q + ((long long)b * a.L + l) * F * F + col;
+  if (j < 0) return;                                  // uniform over the block
+  const float2* src = O + a.obj_off[l] + (long long)a.pos[(l * a.J + j) * 2] * a.obj_w[l] + a.pos[(l * a.J + j) * 2 + 1] + col;
   float2 v[N2];
 #pragma unroll
-  for (int n2 = 0; n2 < N2; ++n2) v[n2] = base[(long long)(t + N1 * n2) * F];
+  for (int n2 = 0; n2 < N2; ++n2) v[n2] = __ldg(src + (long long)(t + N1 * n2) * a.obj_w[l]);
+  stage_ramp<F>(__ldg(sa.delta + (l * a.J + j) * 2), ramp);
   fft_fwd_I2O<F>(v, t, smem + c * Xch<F>::region_cols, a.tw, BlockSync{});
-  const float fx = dft_freq<F>(col);
-  float gyh = 0.f, gyl = 0.f, gxh = 0.f, gxl = 0.f;    // double-float sums of the gradient terms
 #pragma unroll
-  for (int sl = 0; sl < N2; ++sl) {
-    const int k = idxO<F>(t, sl);
-    const float fy = dft_freq<F>(k);
-    float sn, cs;
-    sincospif(2.0f * (fy * dy + fx * dx), &sn, &cs);  // ramp = exp(2 pi i (fy dy + fx dx))
-    const float2 ramp = make_float2(cs, sn);
-    if (!ADJ) {
-      v[sl] = cmul(v[sl], ramp);
-      qb[(long long)k * F] = v[sl];
-    } else {
-      // Re(conj(G) (2 pi i f) Q) = -2 pi f Im(conj(G) Q)
-      const float2 q = qb[(long long)k * F];
-      const float im = fmaf(v[sl].x, q.y, -v[sl].y * q.x);
-      df_add(gyh, gyl, -6.283185307179586f * fy * im);
-      df_add(gxh, gxl, -6.283185307179586f * fx * im);
-      v[sl] = cmulc(v[sl], ramp);
-    }
-  }
-  if (ADJ && sa.dpart) {
-    df_warp_sum(gyh, gyl);
-    df_warp_sum(gxh, gxl);
-    if ((threadIdx.x & 31) == 0) {
-      red[0][threadIdx.x >> 5] = gyh;
-      red[1][threadIdx.x >> 5] = gyl;
-      red[2][threadIdx.x >> 5] = gxh;
-      red[3][threadIdx.x >> 5] = gxl;
-    }
-  }
-  fft_inv_O2I<F>(v, t, smem + c * Xch<F>::region_cols, a.tw, BlockSync{});   // its barriers publish red
+  for (int sl = 0; sl < N2; ++sl) v[sl] = cmul(v[sl], ramp[idxO<F>(t, sl)]);
+  fft_inv_O2I<F>(v, t, smem + c * Xch<F>::region_cols, a.tw, BlockSync{});
+  float2* dst = sa.u + ((long long)b * a.L + l) * F * F + col;
 #pragma unroll
-  for (int n2 = 0; n2 < N2; ++n2) base[(long long)(t + N1 * n2) * F] = v[n2];
-  if (ADJ && sa.dpart && threadIdx.x < 2) {
-    double s = 0.0;
-    for (int w = 0; w < ColCfg<F>::threads / 32; ++w)
-      s += (double)red[2 * threadIdx.x][w] + (double)red[2 * threadIdx.x + 1][w];
-    const double inv = 1.0 / ((double)F * (double)F);
-    sa.dpart[(((long long)(a.batch_off + b) * a.L + l) * gridDim.x + blockIdx.x) * 2 + threadIdx.x] = s * inv;
+  for (int n2 = 0; n2 < N2; ++n2) dst[(t + N1 * n2) * F] = cscale(v[n2], 1.0f / (float)F);
+}
+
+// grid (F/RPB, L, nb)
+template <int F>
+__global__ void __launch_bounds__(RowCfg<F>::threads)
+k_shift_rows(KArgs a, ShiftArgs sa) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int N1 = FftShape<F>::N1, N2 = FftShape<F>::N2, T = RowCfg<F>::T;
+  extern __shared__ float2 smem[];
+  float2* ramp = smem + RowCfg<F>::RPB * Xch<F>::region_rows;
+  const int vec = threadIdx.x / T, t = threadIdx.x % T;
+  const int r = blockIdx.x * RowCfg<F>::RPB + vec, l = blockIdx.y, b = blockIdx.z;
+  const int j = batch_pos(a, a.batch_off + b);
+  if (j < 0) return;                                  // uniform over the block
+  const long long off = (((long long)b * a.L + l) * F + r) * F + t;
+  float2* xc = smem + vec * Xch<F>::region_rows;
+  float2 v[N2];
+#pragma unroll
+  for (int n2 = 0; n2 < N2; ++n2) v[n2] = sa.u[off + N1 * n2];
+  stage_ramp<F>(__ldg(sa.delta + (l * a.J + j) * 2 + 1), ramp);
+  fft_fwd_I2O<F>(v, t, xc, a.tw, WarpSync{});
+#pragma unroll
+  for (int sl = 0; sl < N2; ++sl) v[sl] = cmul(v[sl], ramp[idxO<F>(t, sl)]);
+  fft_inv_O2I<F>(v, t, xc, a.tw, WarpSync{});
+#pragma unroll
+  for (int n2 = 0; n2 < N2; ++n2) sa.patch[off + N1 * n2] = cscale(v[n2], 1.0f / (float)F);
+}
+
+// grid (F/RPB, L, nb)
+template <int F>
+__global__ void __launch_bounds__(RowCfg<F>::threads)
+k_shift_rows_adj(KArgs a, ShiftArgs sa) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int N1 = FftShape<F>::N1, N2 = FftShape<F>::N2, T = RowCfg<F>::T;
+  extern __shared__ float2 smem[];
+  __shared__ float red[2][8];
+  float2* ramp = smem + RowCfg<F>::RPB * Xch<F>::region_rows;
+  const int vec = threadIdx.x / T, t = threadIdx.x % T;
+  const int r = blockIdx.x * RowCfg<F>::RPB + vec, l = blockIdx.y, b = blockIdx.z;
+  const int j = batch_pos(a, a.batch_off + b);
+  double* dx = sa.dpart ? sa.dpart + (((long long)(a.batch_off + b) * a.L + l) * gridDim.x + blockIdx.x) * 2 + 1 : nullptr;
+  if (j < 0) {                                        // uniform over the block
+    if (dx && threadIdx.x == 0) *dx = 0.0;
+    return;
   }
+  const long long off = (((long long)b * a.L + l) * F + r) * F + t;
+  const float2* src = sa.slot + slot_row(sa, b, l, r, F) + t;
+  float2* xc = smem + vec * Xch<F>::region_rows;
+  float2 g[N2];
+#pragma unroll
+  for (int n2 = 0; n2 < N2; ++n2) g[n2] = src[N1 * n2];
+  stage_ramp<F>(__ldg(sa.delta + (l * a.J + j) * 2 + 1), ramp);
+  fft_fwd_I2O<F>(g, t, xc, a.tw, WarpSync{});
+#pragma unroll
+  for (int sl = 0; sl < N2; ++sl) g[sl] = cmulc(g[sl], ramp[idxO<F>(t, sl)]);   // conj(ramp) G: conj of it times U is conj(G) ramp U
+  if (sa.dpart) {
+    float2 v[N2];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) v[n2] = sa.u[off + N1 * n2];
+    fft_fwd_I2O<F>(v, t, xc, a.tw, WarpSync{});
+    float hi = 0.f, lo = 0.f;
+#pragma unroll
+    for (int sl = 0; sl < N2; ++sl)
+      df_add(hi, lo, -6.283185307179586f * dft_freq<F>(idxO<F>(t, sl)) * fmaf(g[sl].x, v[sl].y, -g[sl].y * v[sl].x));
+    const double s = shift_block_sum(hi, lo, red, 1.0 / (double)F);
+    if (threadIdx.x == 0) *dx = s;
+  }
+  fft_inv_O2I<F>(g, t, xc, a.tw, WarpSync{});
+#pragma unroll
+  for (int n2 = 0; n2 < N2; ++n2) sa.g1[off + N1 * n2] = cscale(g[n2], 1.0f / (float)F);
+}
+
+// grid (F/W, L, nb)
+template <int F>
+__global__ void __launch_bounds__(ColCfg<F>::threads)
+k_shift_cols_adj(KArgs a, ShiftArgs sa) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int N1 = FftShape<F>::N1, N2 = FftShape<F>::N2, W = ColCfg<F>::W;
+  extern __shared__ float2 smem[];
+  __shared__ float red[2][8];
+  float2* ramp = smem + W * Xch<F>::region_cols;
+  const int c = threadIdx.x % W, t = threadIdx.x / W;
+  const int col = blockIdx.x * W + c, l = blockIdx.y, b = blockIdx.z;
+  const int j = batch_pos(a, a.batch_off + b);
+  double* dy = sa.dpart ? sa.dpart + (((long long)(a.batch_off + b) * a.L + l) * gridDim.x + blockIdx.x) * 2 : nullptr;
+  if (j < 0) {                                        // uniform over the block
+    if (dy && threadIdx.x == 0) *dy = 0.0;
+    return;
+  }
+  const long long off = ((long long)b * a.L + l) * F * F + col;
+  float2* xc = smem + c * Xch<F>::region_cols;
+  float2 g[N2];
+#pragma unroll
+  for (int n2 = 0; n2 < N2; ++n2) g[n2] = sa.g1[off + (t + N1 * n2) * F];
+  stage_ramp<F>(__ldg(sa.delta + (l * a.J + j) * 2), ramp);
+  fft_fwd_I2O<F>(g, t, xc, a.tw, BlockSync{});
+  if (sa.dpart) {
+    float2 v[N2];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) v[n2] = sa.u[off + (t + N1 * n2) * F];
+    fft_fwd_I2O<F>(v, t, xc, a.tw, BlockSync{});
+    float hi = 0.f, lo = 0.f;
+#pragma unroll
+    for (int sl = 0; sl < N2; ++sl)
+      df_add(hi, lo, -6.283185307179586f * dft_freq<F>(idxO<F>(t, sl)) * fmaf(g[sl].x, v[sl].y, -g[sl].y * v[sl].x));
+    const double s = shift_block_sum(hi, lo, red, 1.0 / (double)F);
+    if (threadIdx.x == 0) *dy = s;
+  }
+#pragma unroll
+  for (int sl = 0; sl < N2; ++sl) g[sl] = cmulc(g[sl], ramp[idxO<F>(t, sl)]);
+  fft_inv_O2I<F>(g, t, xc, a.tw, BlockSync{});
+  float2* dst = sa.slot + slot_row(sa, b, l, 0, F) + col;
+  const int stride = sa.slot_pair ? 2 * F : F;
+#pragma unroll
+  for (int n2 = 0; n2 < N2; ++n2) dst[(long long)(t + N1 * n2) * stride] = cscale(g[n2], 1.0f / (float)F);
 }
 
 // Position gradient: g_delta[l][j][a] = sum, in call-entry order, of the partials of every
-// entry i with bidx[i] = j; 0 for positions outside the call.   grid (ceil(L*J/256))
+// entry i with bidx[i] = j; 0 for positions outside the call.   grid (ceil(L*J/8))
 __global__ void k_delta_grad(const int32_t* __restrict__ bidx, int nbatch, int L, int J, const double* __restrict__ dpart,
                              int nstrips, float* __restrict__ g_delta);
 
