@@ -188,10 +188,13 @@ namespace {
 // wavelengths with 32 / 58 / 80 / 134 positions per batch (400 in all) 2.48 / 2.29 / 2.28 / 2.13 ms,
 // 256^2 x 4 x 3 with 50 / 68 / 100 / 134 3.18 / 3.13 / 3.06 / 3.00 ms: so the target is in elements.
 // One field per position: 64^2 with 22 / 32 / 64 of 64 positions 139 / 117 / 98 us (launches), 128^2
-// with 68 / 134 / 200 / 400 of 400 positions 262 / 243 / 235 / 241 us.
+// with 68 / 134 / 200 / 400 of 400 positions 262 / 243 / 235 / 241 us; 256^2 x 6 modes x 2 wavelengths
+// with 10 / 13 of 25 positions 311 / 283 us.  So batches of under kSmallBatchElems are merged.  A chirp-z
+// element counts for four (two transforms of 2 F points per axis, bound by arithmetic: short batches lose
+// little and their overlap fills the tails): 64^2 x 5 x 2 with 151 / 51 of 151 positions 556 / 507 us.
 constexpr long long kMaxScratch = 8ll << 30;   // default upper bound of one buffer set
 constexpr long long kBatchElems = 320ll << 20; // field elements per batch the default aims for (1200 of 512^2)
-constexpr long long kSmallBatchElems = 4ll << 20;
+constexpr long long kSmallBatchElems = 8ll << 20;
 constexpr long long kMinBatchPositions = 64;   // at least this many positions (when they fit)
 constexpr long long kMinBatches = 3;           // batches per call (overlap), when they are not small
 constexpr long long kBatchRows = 32768;        // and at least this many 1D FFT rows per pass
@@ -593,7 +596,8 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
       const long long evals = std::max(target.evals, (target.elems + F * F - 1) / (F * F));
       B = std::min<long long>(B, std::max({(evals + LM - 1) / LM, (kBatchRows + LM * F - 1) / (LM * F),
                                            target.min_positions}));
-      const long long nmin = std::max<long long>(1, std::min<long long>(kMinBatches, g->J * elems / kSmallBatchElems));
+      const long long work = g->J * elems * (g->zoom ? 4 : 1);
+      const long long nmin = std::max<long long>(1, std::min<long long>(kMinBatches, work / kSmallBatchElems));
       B = std::min<long long>(B, std::max<long long>(1, (g->J + nmin - 1) / nmin));
     }
     p->B = (int)std::max<long long>(1, std::min<long long>(B, ptycho::kMaxB));
