@@ -142,6 +142,8 @@ k_shift_rows_adj(KArgs a, ShiftArgs sa) {
   pdl_wait();
   pdl_trigger();
   constexpr int N1 = FftShape<F>::N1, N2 = FftShape<F>::N2, T = RowCfg<F>::T;
+  static_assert(RowCfg<F>::RPB == ColCfg<F>::W && RowCfg<F>::threads == 256 && ColCfg<F>::threads == 256,
+                "both adjoint passes leave F/W partials per window, from blocks of eight warps");
   extern __shared__ float2 smem[];
   __shared__ float red[2][8];
   float2* ramp = smem + RowCfg<F>::RPB * Xch<F>::region_rows;

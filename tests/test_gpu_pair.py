@@ -10,7 +10,8 @@ import pytest
 import torch
 
 from synthetic import workloads as syn
-from test_gpu_parity import Case, assert_ok, check_all, dev, max_rel, strong_z  # noqa: F401
+from test_gpu_parity import (Case, _assert_offsets_ok, _offset_errors, _offsets, assert_ok, check_all, dev,  # noqa: F401
+                             max_rel, strong_z)
 
 pytestmark = pytest.mark.gpu
 
@@ -82,4 +83,18 @@ def test_a_bad_position_index_leaves_its_partner_alone(dev, F, M, bad):
     for x, y in zip(a[1:], b[1:]):
         assert np.isfinite(x.cpu().numpy()).all()
         assert max_rel(x.cpu().numpy(), y.cpu().numpy()) < GRAD_REORDERED
+    plan.close()
+
+
+# fractional offsets of several pixels and of exactly none, one mode and several, an odd batch (the last
+# position's lane of the scratch slot) and positions taken one by one (the one-field slot)
+@pytest.mark.parametrize("F,L,M,B", [(64, 2, 1, 9), (128, 1, 3, 3), (256, 1, 2, 1), (512, 1, 2, 2)])
+def test_shift_by_axes(dev, F, L, M, B):
+    case = _case(dev, F, L, M, 3, 90 + F + B)
+    delta = _offsets(case.w, F + B, amp=2.5)
+    delta[0, 2] = 0.0
+    delta[0, 3, 1] = 0.0
+    plan = case.plan(scratch_bytes=B * L * M * F * F * 8)
+    _assert_offsets_ok(_offset_errors(case, plan, delta))
+    _assert_offsets_ok(_offset_errors(case, plan, delta, [8, 0, 5]))
     plan.close()
