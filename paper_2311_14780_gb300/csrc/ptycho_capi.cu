@@ -17,15 +17,19 @@ namespace ptycho {
 // Fixed-order FP64 sum of the per-block loss partials: one cluster of kReduceBlocks blocks, whose sums the
 // first block adds in block order through distributed shared memory.  FP64 additions bound it (two per
 // clock and SM on this part), so it wants several SMs: 102 400 partials (400 frames of 512^2) took 49 us
-// in one block of 256 threads, 36 us in one of 1024.
+// in one block of 256 threads, 36 us in one of 1024.  A block's shared memory may be written from another
+// one only once it has started, which the first phase of the cluster's barrier says: arrived at on entry,
+// waited for after the block's own sum, so that it costs no time of its own.
 __global__ void __cluster_dims__(kReduceBlocks, 1, 1) __launch_bounds__(kReduceThreads)
 k_loss_reduce(const double* __restrict__ part, long long n, double* out) {
-  pdl_wait();
   __shared__ double red[kReduceThreads / 32];
   __shared__ double sums[kReduceBlocks];
   const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   const int rank = (int)cl.block_rank();
+  cl.barrier_arrive();
+  pdl_wait();
   const double s = block_sum_partials(part, n, rank * kReduceThreads + (int)threadIdx.x, kReduceBlocks * kReduceThreads, red);
+  cl.barrier_wait();                                  // every block of the cluster runs
   if (threadIdx.x == 0) *cl.map_shared_rank(&sums[rank], 0) = s;
   cl.sync();
   if (rank == 0 && threadIdx.x == 0) {
