@@ -91,6 +91,12 @@ __device__ __forceinline__ cpair ld_pair(const float4* p) {
 }
 __device__ __forceinline__ void st_pair(float4* p, cpair v) { *p = make_float4(v.re.x, v.re.y, v.im.x, v.im.y); }
 
+// The bounded wait of a whole warp, with one outcome for its lanes: a lane whose wait ran out must not leave
+// alone, the others' warp-wide exchanges and shuffles count on it.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t phase, int* status) {
+  return __all_sync(0xffffffffu, mbar_wait_bounded(bar, phase, status));
+}
+
 // Element index of slot i of thread t in spectrum order (layout O of fft_regs.cuh; at F = 512
 // t + 32 i).  Natural order is t + T i.
 template <int F> __device__ __forceinline__ int pidxO(int t, int i) {
@@ -356,7 +362,7 @@ k_row_fwd_p(const float2* __restrict__ O, const float2* __restrict__ P, float4* 
     if (more) pp = pair_pos(a, p + step, l);
     float4* out = S + (((long long)p * a.C + l * M) * F + r) * F;
     for (int m = 0; m < M; ++m, out += F * F) {
-      if (!mbar_wait_bounded(pbar, phase, a.status)) return;
+      if (!mbar_wait_warp(pbar, phase, a.status)) return;
       phase ^= 1;
       cpair x[16];
 #pragma unroll
@@ -598,6 +604,28 @@ __host__ __device__ constexpr int row_adj_p_smem(int M, int rpb) {
 // in as many blocks as that makes.
 constexpr int row_adj_p_feeders(int ct) { return ct <= 160 ? 1 : 2; }
 
+// Whether every one of the block's NPW feeding warps agrees (their threads only, all of them); what any of
+// them read from shared memory before, it has read.  A wait that ran out for one thread must end the loop
+// of all: the others would stand at a barrier that nobody else comes to.
+template <int NPW>
+__device__ __forceinline__ bool feeders_agree(bool ok) {
+  __syncwarp();
+  ok = __all_sync(0xffffffffu, ok);
+  if constexpr (NPW > 1) {
+    uint32_t all;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(all)
+        : "r"((uint32_t)ok), "n"(32 * NPW)
+        : "memory");
+    ok = all != 0;
+  }
+  return ok;
+}
+
 // Next pair of this split after p with a valid position, or -1 (uniform over the block).
 __device__ __forceinline__ int next_pair(const int2* spos, int p, int nb, int nsplit) {
   for (int q = p + nsplit; 2 * q < nb; q += nsplit)
@@ -666,9 +694,9 @@ k_row_adj_p(const float2* __restrict__ O, const float2* __restrict__ P, float4* 
     if (pn >= 0) fetch(pn, 1);
     for (int k = 0; p >= 0; ++k) {
       const int buf = k & 1;
-      if (!mbar_wait_bounded(&done[buf], (k >> 1) & 1, a.status)) break;
+      const bool ok = mbar_wait_bounded(&done[buf], (k >> 1) & 1, a.status);
       float4* dst = S + (((long long)p * a.C + l * M) * F + row0) * F;  // the block's rows, contiguous
-      for (int rr = 0; rr < rpb; ++rr) {
+      for (int rr = 0; rr < (ok ? rpb : 0); ++rr) {
         const float4* red = Sst + (buf * V + rr * M) * VEC + pt;
 #pragma unroll 4
         for (int i = 0; i < F / NPT; ++i) {
@@ -683,9 +711,8 @@ k_row_adj_p(const float2* __restrict__ O, const float2* __restrict__ P, float4* 
         }
       }
       const int p2 = pn >= 0 ? next_pair(spos, pn, a.nb, nsplit) : -1;
+      if (!feeders_agree<NPW>(ok)) break;             // and every feeder has read the buffer
       if (p2 >= 0) {
-        if constexpr (NPW > 1) asm volatile("bar.sync 1, %0;" ::"n"(NPT) : "memory");
-        else __syncwarp();                            // every feeder has read the buffer
         fence_proxy_async_smem();
         fetch(p2, buf);
       }
@@ -705,7 +732,7 @@ k_row_adj_p(const float2* __restrict__ O, const float2* __restrict__ P, float4* 
   }
   for (int k = 0; p >= 0; ++k, p = next_pair(spos, p, a.nb, nsplit)) {
     const int buf = k & 1;
-    if (!mbar_wait_bounded(&full[buf], (k >> 1) & 1, a.status)) return;
+    if (!mbar_wait_warp(&full[buf], (k >> 1) & 1, a.status)) return;
     const bool v0 = spos[2 * p].x >= 0, v1 = 2 * p + 1 < a.nb && spos[2 * p + 1].x >= 0;
     float4* reg = Sst + (buf * V + vec) * VEC;
     const Place<F, false> pl(reinterpret_cast<char*>(reg), 0, t, pair_n1<F>(t), t);
@@ -802,7 +829,7 @@ k_row_adj_p1(const float2* __restrict__ O, const float2* __restrict__ P, float4*
   for (int k = 0; p < np; ++k, p += nsplit) {
     const int buf = k & 1;
     const PairPos pn = pair_pos(a, min(p + nsplit, np - 1), l);
-    if (!mbar_wait_bounded(&full[buf], (k >> 1) & 1, a.status)) return;
+    if (!mbar_wait_warp(&full[buf], (k >> 1) & 1, a.status)) return;
     float4* reg = Sst + (buf * VPW + vec) * VEC;
     const Place<F, false> pl(reinterpret_cast<char*>(reg), 0, t, pair_n1<F>(t), t);
     cpair x[16];
@@ -816,7 +843,7 @@ k_row_adj_p1(const float2* __restrict__ O, const float2* __restrict__ P, float4*
       fence_proxy_async_smem();
       fetch(p + 2 * nsplit, buf);
     }
-    if (!mbar_wait_bounded(&obar, k & 1, a.status)) return;
+    if (!mbar_wait_warp(&obar, k & 1, a.status)) return;
     const bool v0 = pp.yx[0].x >= 0, v1 = pp.yx[1].x >= 0;
     float2* go = reinterpret_cast<float2*>(S + (((long long)p * a.C + l) * F + r) * F) + t;
 #pragma unroll

@@ -40,3 +40,25 @@ def test_another_blocks_shared_memory_only_after_a_cluster_barrier():
     for name, body in users:
         before = body[:body.index("map_shared_rank")]
         assert re.search(r"\.(barrier_wait|sync)\s*\(", before), name
+
+
+def test_no_thread_leaves_a_loop_by_its_own_wait():
+    """The outcome of a bounded wait differs between threads when it runs out just as the copy lands, so
+    it is agreed on (by the warp, the feeding warps or the block) before it decides about an exit: whoever
+    stays would wait for those who left at the next barrier or shuffle, which has no limit."""
+    for name, body in [(n, b) for _, n, b in _kernels() if "mbar_wait_bounded" in b]:
+        for m in re.finditer(r"mbar_wait_bounded", body):
+            start = max(body.rfind(c, 0, m.start()) for c in ";{}") + 1
+            stmt = body[start:body.index(";", m.end()) + 1]
+            tail = body[body.index(";", m.end()):]
+            agreed = re.search(r"__syncthreads_and\s*\(\s*mbar_wait_bounded", stmt)
+            kept = re.search(r"[^=!<>]=[^=]", stmt.split("mbar_wait_bounded")[0])
+            alone = not re.search(r"\b(return|break)\b", stmt) and (not kept or re.search(r"feeders_agree<\w+>\(ok\)", tail))
+            assert agreed or alone, (name, stmt.strip())
+
+
+def test_named_barriers_carry_the_outcome():
+    """A barrier among some of a block's warps is one that also says whether all of them go on."""
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh")):
+            assert not re.search(r"bar(rier)?\.(cta\.)?sync", _source(f)), f
