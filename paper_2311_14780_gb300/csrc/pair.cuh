@@ -97,6 +97,12 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t phase, in
   return __all_sync(0xffffffffu, mbar_wait_bounded(bar, phase, status));
 }
 
+// A give-up's last look at a copy that may still be under way (fetch i of those that go round two buffers, one
+// phase each time): a bounded chance to land before the block's shared memory goes to another one.
+__device__ __forceinline__ void drain_fetch(uint64_t* bar, int i, int* status) {
+  mbar_wait_bounded(&bar[i & 1], (i >> 1) & 1, status);
+}
+
 // Element index of slot i of thread t in spectrum order (layout O of fft_regs.cuh; at F = 512
 // t + 32 i).  Natural order is t + T i.
 template <int F> __device__ __forceinline__ int pidxO(int t, int i) {
@@ -362,7 +368,10 @@ k_row_fwd_p(const float2* __restrict__ O, const float2* __restrict__ P, float4* 
     if (more) pp = pair_pos(a, p + step, l);
     float4* out = S + (((long long)p * a.C + l * M) * F + r) * F;
     for (int m = 0; m < M; ++m, out += F * F) {
-      if (!mbar_wait_warp(pbar, phase, a.status)) return;
+      if (!mbar_wait_warp(pbar, phase, a.status)) {
+        mbar_wait_bounded(pbar, phase, a.status);     // the only copy under way
+        return;
+      }
       phase ^= 1;
       cpair x[16];
 #pragma unroll
@@ -711,7 +720,11 @@ k_row_adj_p(const float2* __restrict__ O, const float2* __restrict__ P, float4* 
         }
       }
       const int p2 = pn >= 0 ? next_pair(spos, pn, a.nb, nsplit) : -1;
-      if (!feeders_agree<NPW>(ok)) break;             // and every feeder has read the buffer
+      if (!feeders_agree<NPW>(ok)) {                  // (else every feeder has read the buffer)
+        drain_fetch(full, k, a.status);
+        if (pn >= 0) drain_fetch(full, k + 1, a.status);
+        break;
+      }
       if (p2 >= 0) {
         fence_proxy_async_smem();
         fetch(p2, buf);
@@ -732,6 +745,7 @@ k_row_adj_p(const float2* __restrict__ O, const float2* __restrict__ P, float4* 
   }
   for (int k = 0; p >= 0; ++k, p = next_pair(spos, p, a.nb, nsplit)) {
     const int buf = k & 1;
+    // (the feeding warps, which find done[buf] incomplete then, see to the copies under way)
     if (!mbar_wait_warp(&full[buf], (k >> 1) & 1, a.status)) return;
     const bool v0 = spos[2 * p].x >= 0, v1 = 2 * p + 1 < a.nb && spos[2 * p + 1].x >= 0;
     float4* reg = Sst + (buf * V + vec) * VEC;
@@ -826,10 +840,18 @@ k_row_adj_p1(const float2* __restrict__ O, const float2* __restrict__ P, float4*
     pr[i] = __ldg(P + row + T * i);
     acc[i] = make_float2(0.f, 0.f);
   }
+  // what a give-up at pair k leaves under way: scratch rows from fetch i on, the object rows of pair k
+  auto drain = [&](int i, int k) {
+    for (int q = i; q < i + 2 && split + q * nsplit < np; ++q) drain_fetch(full, q, a.status);
+    mbar_wait_bounded(&obar, k & 1, a.status);
+  };
   for (int k = 0; p < np; ++k, p += nsplit) {
     const int buf = k & 1;
     const PairPos pn = pair_pos(a, min(p + nsplit, np - 1), l);
-    if (!mbar_wait_warp(&full[buf], (k >> 1) & 1, a.status)) return;
+    if (!mbar_wait_warp(&full[buf], (k >> 1) & 1, a.status)) {
+      drain(k, k);
+      return;
+    }
     float4* reg = Sst + (buf * VPW + vec) * VEC;
     const Place<F, false> pl(reinterpret_cast<char*>(reg), 0, t, pair_n1<F>(t), t);
     cpair x[16];
@@ -843,7 +865,10 @@ k_row_adj_p1(const float2* __restrict__ O, const float2* __restrict__ P, float4*
       fence_proxy_async_smem();
       fetch(p + 2 * nsplit, buf);
     }
-    if (!mbar_wait_warp(&obar, k & 1, a.status)) return;
+    if (!mbar_wait_warp(&obar, k & 1, a.status)) {
+      drain(k + 1, k);
+      return;
+    }
     const bool v0 = pp.yx[0].x >= 0, v1 = pp.yx[1].x >= 0;
     float2* go = reinterpret_cast<float2*>(S + (((long long)p * a.C + l) * F + r) * F) + t;
 #pragma unroll

@@ -62,3 +62,19 @@ def test_named_barriers_carry_the_outcome():
     for f in sorted(os.listdir(CSRC)):
         if f.endswith((".cu", ".cuh")):
             assert not re.search(r"bar(rier)?\.(cta\.)?sync", _source(f)), f
+
+
+def test_an_exit_waits_for_its_copies():
+    """Every warp that issues asynchronous copies gives those under way a bounded chance to land before it
+    gives up: a copy that lands later writes into shared memory that belongs to another block by then."""
+    issues = re.compile(r"bulk_load\s*\(|tma_load_2d\s*\(|tma_issue<\w+>\s*\(|pair_tile_issue<\w+>\s*\(|fetch_probe\s*\(")
+    for name, body in [(n, b) for _, n, b in _kernels() if issues.search(b) and "mbar_wait" in b]:
+        for m in re.finditer(r"if \(!(mbar_wait_warp|feeders_agree)[^{;]*([{;])", body):
+            if m.group(2) == "{":
+                block = body[m.end():body.index("}", m.end())]
+                assert re.search(r"mbar_wait_bounded|drain", block), (name, m.group(0))
+            else:                                      # a warp that issues none: its block's feeders drain
+                assert re.search(r"if \(!feeders_agree<\w+>\(ok\)\) {\s*drain_fetch", body), (name, m.group(0))
+        if "__syncthreads_and" in body:
+            after = body[body.index("__syncthreads_and"):]
+            assert re.search(r"if \((threadIdx\.x == 0|!ok)[^;]*\)?\s*mbar_wait_bounded", after), name
