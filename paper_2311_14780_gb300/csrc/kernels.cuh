@@ -506,8 +506,9 @@ __device__ __forceinline__ void df_warp_sum(float& hi, float& lo) {
 // instructions per pixel at two per cycle and SM, DRAM 12 % busy), hence the compile-time REMAP and ONE
 // (one intensity slice) and one reduction per position by one warp.
 // The loss terms of a block are summed as double-floats: per thread, then, for each position, by one warp
-// over the block's threads in a fixed order into one partial per (call entry, block); the sigma- and
-// z-gradient terms per thread, by a warp tree and in FP64 over the eight warps.
+// over the threads of each of the block's eight warps; their sums in FP64 (a double-float holds 48 bits), in a
+// fixed order, into one partial per (call entry, block).  The sigma- and z-gradient terms per thread, by a warp
+// tree and in FP64 over the eight warps.
 // grid (F*F/(kLossThreads*kLossPx), ceil(nb / la.npos))
 struct LossShared {
   float2 sum[kLossPosMax][kLossThreads];              // loss terms (hi, lo) of each thread
@@ -638,14 +639,23 @@ __device__ __forceinline__ void loss_positions_body(const KArgs& a, const LossAr
     static_assert(kLossPosMax <= NW, "one warp per position");
     const int n = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (n < nb) {
-      float2 v = sm.sum[n][lane];
+      // lane i: threads 8 i ... 8 i + 7 (from a different one on each, for the banks), so that four lanes
+      // hold a warp's
+      float2 v = sm.sum[n][8 * lane + (lane & 7)];
 #pragma unroll
-      for (int i = 1; i < NW; ++i) {
-        const float2 u = sm.sum[n][lane + 32 * i];
+      for (int i = 1; i < 8; ++i) {
+        const float2 u = sm.sum[n][8 * lane + ((lane + i) & 7)];
         df_add_df(v.x, v.y, u.x, u.y);
       }
-      df_warp_sum(v.x, v.y);
-      if (lane == 0) la.loss_part[part + (long long)n * NB] = (double)v.x + (double)v.y;
+#pragma unroll
+      for (int o = 1; o < 4; o *= 2) {
+        const float uh = __shfl_xor_sync(0xffffffffu, v.x, o), ul = __shfl_xor_sync(0xffffffffu, v.y, o);
+        df_add_df(v.x, v.y, uh, ul);
+      }
+      double s = (double)v.x + (double)v.y;
+#pragma unroll
+      for (int o = 4; o < 32; o *= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) la.loss_part[part + (long long)n * NB] = s;
     }
   }
   if (la.sig_part || la.z_part) {

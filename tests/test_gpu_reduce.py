@@ -38,3 +38,24 @@ def test_loss_of_repeated_frames(stack, n):
     assert len(set(got)) == 1
     assert abs(got[0] / (n * one) - 1) <= 4 * n * 2.0 ** -53
     assert plan.status() == 0
+
+
+# positions per block of the loss pass: one (few of 64^2) and eight (83 of 256^2), the last group of three;
+# the frame's place in its group
+@pytest.mark.parametrize("F,J,j", [(64, 3, 0), (64, 3, 2), (256, 83, 0), (256, 83, 7), (256, 83, 8), (256, 83, 82)])
+def test_loss_keeps_64_bits_over_a_block(F, J, j):
+    """Terms of three warps of a block that FP64 adds exactly and a double-float (two FP32 numbers) cannot
+    hold: 2^36 + 2^10 + 2^-16.  A zero probe leaves the background alone; every other term is zero."""
+    from paper_2311_14780_gb300 import Plan
+    dev = torch.device("cuda", 0)
+    plan = Plan(F, 1, 1, J, [(F, F)], np.zeros((1, J, 2), np.int32), scratch_bytes=(J + 1) * F * F * 8)
+    bg = torch.ones(F, F)
+    flat = bg.view(-1)
+    flat[0], flat[128], flat[256] = 2.0 ** 36, 2.0 ** 10, 2.0 ** -16
+    Im = bg.repeat(J, 1, 1)
+    Im[j].view(-1)[[0, 128, 256]] = 0.0
+    O = torch.ones(F * F, dtype=torch.complex64, device=dev)
+    P = torch.zeros(1, 1, F, F, dtype=torch.complex64, device=dev)
+    got = plan.loss(O, P, Im.to(dev), bg=bg.to(dev))
+    assert float(got.item()) == 2.0 ** 36 + 2.0 ** 10 + 2.0 ** -16
+    plan.close()
