@@ -360,6 +360,15 @@ int ptycho_step_host(ptycho_plan_t* plan, ptycho_adam_t* state, float* O, float*
 
 /* Number of kernel launches issued by the most recent compute call on this plan. */
 int64_t ptycho_plan_last_launches(const ptycho_plan_t* plan);
+/* What the plan chose for its calls; -1 for a null plan or an unknown ``what``.
+ * PAIR_PASSES: 1 if they transform pairs of positions (see the pipeline variants), else 0.
+ * BATCH_POSITIONS: positions per batch.  ROW_ADJ_SPLITS: position splits of the row adjoint over all modes of
+ * a wavelength (each with its own probe gradient).  COLUMN_GROUPS: mode groups of the column passes. */
+#define PTYCHO_QUERY_PAIR_PASSES 0
+#define PTYCHO_QUERY_BATCH_POSITIONS 1
+#define PTYCHO_QUERY_ROW_ADJ_SPLITS 2
+#define PTYCHO_QUERY_COLUMN_GROUPS 3
+int64_t ptycho_plan_query(const ptycho_plan_t* plan, int what);
 
 /* Device-side status of the plan since the previous query, then cleared.  Bit 0
  * (PTYCHO_STATUS_BAD_INDEX): a batch_idx entry was outside [0, J); that position was

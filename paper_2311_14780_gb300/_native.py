@@ -62,6 +62,7 @@ SIGNATURES = [
     ("ptycho_plan_numel_O", ctypes.c_int64, [_VP]),
     ("ptycho_plan_numel_P", ctypes.c_int64, [_VP]),
     ("ptycho_plan_last_launches", ctypes.c_int64, [_VP]),
+    ("ptycho_plan_query", ctypes.c_int64, [_VP, ctypes.c_int]),
     ("ptycho_forward", _I, [_VP, _VP, _VP, _VP, _VP, _VP, _VP]),
     ("ptycho_loss", _I, [_VP, _VP, _VP, _VP, _VP, _VP, _VP, _I, _VP, _I, _VP, _VP]),
     ("ptycho_adjoint", _I, [_VP, _VP, _VP, _VP, _VP, _VP, _VP, _I, _VP, _I, _VP, _VP, _VP, _VP]),

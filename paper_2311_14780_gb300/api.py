@@ -146,6 +146,10 @@ class Plan:
     def last_launches(self) -> int:
         return int(_native.lib().ptycho_plan_last_launches(self._h_plan))
 
+    def query(self, what: int) -> int:
+        """ptycho_plan_query: what the plan chose for its calls (PTYCHO_QUERY_* in include/ptycho.h)."""
+        return int(_native.lib().ptycho_plan_query(self._h_plan, int(what)))
+
     def profile(self, enable: bool = True):
         """Start (or stop) per-kernel event timing of this plan's launches."""
         _check(_native.lib().ptycho_plan_profile(self._h_plan, 1 if enable else 0), "ptycho_plan_profile")

@@ -891,6 +891,16 @@ int64_t ptycho_plan_workspace_bytes(const ptycho_plan_t* p) { return p ? p->byte
 int64_t ptycho_plan_numel_O(const ptycho_plan_t* p) { return p ? p->O_numel : 0; }
 int64_t ptycho_plan_numel_P(const ptycho_plan_t* p) { return p ? p->P_numel : 0; }
 int64_t ptycho_plan_last_launches(const ptycho_plan_t* p) { return p ? p->last_launches : 0; }
+int64_t ptycho_plan_query(const ptycho_plan_t* p, int what) {
+  if (!p) return -1;
+  switch (what) {
+    case PTYCHO_QUERY_PAIR_PASSES: return p->pair;
+    case PTYCHO_QUERY_BATCH_POSITIONS: return p->B;
+    case PTYCHO_QUERY_ROW_ADJ_SPLITS: return p->pair || p->adj_l ? p->nsplit_adj : 1;
+    case PTYCHO_QUERY_COLUMN_GROUPS: return p->G;
+    default: return -1;
+  }
+}
 
 int ptycho_plan_profile(ptycho_plan_t* p, int enable) {
   if (!p) return PTYCHO_EINVAL;

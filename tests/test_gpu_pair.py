@@ -98,3 +98,49 @@ def test_shift_by_axes(dev, F, L, M, B):
     _assert_offsets_ok(_offset_errors(case, plan, delta))
     _assert_offsets_ok(_offset_errors(case, plan, delta, [8, 0, 5]))
     plan.close()
+
+
+PAIR_PASSES, BATCH_POSITIONS, ROW_ADJ_SPLITS, COLUMN_GROUPS = range(4)      # PTYCHO_QUERY_* of include/ptycho.h
+
+
+# the counts beside each line of the rule: one field per position by frame size, modes that fill whole warps
+# of a block of 320 threads and the next that do not, one position per batch, flags
+@pytest.mark.parametrize("F,L,M,B,flags,pair", [
+    (64, 1, 1, 9, 0, 1), (128, 1, 1, 9, 0, 1), (256, 1, 1, 9, 0, 0), (512, 1, 1, 9, 0, 0), (256, 2, 1, 9, 0, 1),
+    (512, 2, 1, 9, 0, 1), (512, 1, 10, 2, 0, 1), (512, 1, 11, 2, 0, 0), (256, 1, 11, 4, 0, 0), (256, 1, 20, 4, 0, 1),
+    (128, 1, 40, 4, 0, 1), (64, 1, 80, 4, 0, 1), (64, 1, 88, 4, 0, 0), (256, 1, 4, 1, 0, 0), (256, 1, 4, 3, 0, 1),
+    (256, 1, 4, 4, ONE_FIELD, 0), (256, 1, 4, 4, 512, 1)])
+def test_which_plans_take_the_pair_passes(dev, F, L, M, B, flags, pair):
+    from paper_2311_14780_gb300 import Plan
+    plan = Plan(F, L, M, 9, [(F, F)] * L, np.zeros((L, 9, 2), np.int32), scratch_bytes=B * L * M * F * F * 8, flags=flags)
+    assert plan.query(PAIR_PASSES) == pair
+    assert plan.query(BATCH_POSITIONS) == (B - B % 2 if pair else B)   # whole pairs within the budget
+    plan.close()
+
+
+# as many modes as a block of the pair row adjoint takes
+@pytest.mark.parametrize("F,M", [(256, 18), (256, 20), (128, 40), (64, 72), (64, 80)])
+def test_many_modes(dev, F, M):
+    case = _case(dev, F, 1, M, 3, 60 + F + M)
+    plan = case.plan()
+    assert plan.query(PAIR_PASSES) == 1
+    assert_ok(check_all(case, plan))
+    assert_ok(check_all(case, plan, frames=[8, 1, 5]))
+    plan.close()
+
+
+@pytest.mark.parametrize("F,L,M", [(64, 2, 1), (64, 1, 80), (128, 2, 5), (128, 1, 1), (256, 1, 3), (256, 2, 10), (512, 2, 1),
+                                   (512, 1, 10)])
+def test_patterns_and_loss_are_the_one_field_passes_bit_by_bit(dev, F, L, M):
+    """With the same positions per batch and one mode group."""
+    case = _case(dev, F, L, M, 3, 70 + F + M)
+    kw = dict(scratch_bytes=4 * L * M * F * F * 8, col_groups=1)
+    plan, ref = case.plan(**kw), case.plan(flags=ONE_FIELD, **kw)
+    assert (plan.query(PAIR_PASSES), ref.query(PAIR_PASSES)) == (1, 0)
+    assert all(p.query(BATCH_POSITIONS) == 4 and p.query(COLUMN_GROUPS) == 1 for p in (plan, ref))
+    args = (case.O, case.P, case.sig_t, case.bg_t)
+    assert torch.equal(plan.forward(*args), ref.forward(*args))
+    loss = [p.loss(case.O, case.P, case.Im, case.sig_t, case.bg_t, case.mask_t) for p in (plan, ref)]
+    assert torch.equal(*loss)
+    plan.close()
+    ref.close()
