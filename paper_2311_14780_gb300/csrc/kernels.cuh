@@ -57,6 +57,7 @@ struct KArgs {
   int chunk_base, chunk_len;     // global modes [chunk_base, chunk_base + chunk_len)
   int MG;                        // modes per column-kernel group
   int G;                         // groups per chunk (Ipart has G slices per position)
+  int deal;                      // positions dealt to a split of the fused row passes at a time (1 or 2)
   int* status;                   // device status word (bit 0: a position index was out of range)
   int box[kMaxL][4];             // per wavelength: rows [box0, box2) x cols [box1, box3) covered by
                                  // the batch's patches (the whole object when not known on the host)
@@ -1230,14 +1231,17 @@ __device__ __forceinline__ void acc_conjmul(float2& acc, float2 o, float2 v) {
   acc.y = fmaf(o.x, v.y, fmaf(-o.y, v.x, acc.y));
 }
 
-// Positions are dealt to the splits in pairs (2p, 2p + 1), p = split, split + nsplit, ..., the order of
-// the pair passes.  Next position of this split after b whose index is valid, or -1 (uniform over the
-// block); before_split(split, nsplit) comes before the first.
-__device__ __forceinline__ int before_split(int split, int nsplit) { return 2 * (split - nsplit) + 1; }
-__device__ __forceinline__ int next_pos(const int2* spos, int b, int nb, int nsplit) {
-  do b = (b & 1) ? 2 * ((b >> 1) + nsplit) : b + 1;
-  while (b < nb && spos[b].x < 0);
-  return b < nb ? b : -1;
+// Positions are dealt to the splits in groups of a.deal: one by one, so that every split gets its share of
+// a short batch, or two by two, the order of the pair passes (which the shared launches of a plan with those
+// follow).  Next position of this split after b whose index is valid, or -1 (uniform over the block);
+// before_split(a, split, nsplit) comes before the first.
+__device__ __forceinline__ int before_split(const KArgs& a, int split, int nsplit) {
+  return a.deal * (split - nsplit + 1) - 1;
+}
+__device__ __forceinline__ int next_pos(const KArgs& a, const int2* spos, int b, int nsplit) {
+  do b += (b & (a.deal - 1)) == a.deal - 1 ? 1 + a.deal * (nsplit - 1) : 1;
+  while (b < a.nb && spos[b].x < 0);
+  return b < a.nb ? b : -1;
 }
 
 // Copies of the rpb object rows of position (y, x) (8-byte pieces: x may be odd).
@@ -1293,12 +1297,12 @@ __device__ __forceinline__ void row_adj_l_body(const float2* __restrict__ O, con
   float2 acc[N2];
 #pragma unroll
   for (int n2 = 0; n2 < N2; ++n2) acc[n2] = make_float2(0.f, 0.f);
-  int b = next_pos(spos, before_split(split, nsplit), a.nb, nsplit);
+  int b = next_pos(a, spos, before_split(a, split, nsplit), nsplit);
   if (b >= 0) prefetch(b, 0);
   for (int buf = 0; b >= 0; buf ^= 1) {
     cp_async_wait<0>();
     __syncthreads();                                  // position b has landed; buffer buf^1 is free
-    const int bn = next_pos(spos, b, a.nb, nsplit);
+    const int bn = next_pos(a, spos, b, nsplit);
     if (bn >= 0) prefetch(bn, buf ^ 1);
     const float s = ssig[b];
     float2* reg = Sst + (buf * V + vec) * RR;         // this vector's row, then its exchange/mode-sum area
@@ -1398,12 +1402,12 @@ __device__ __forceinline__ void row_adj_w_body(const float2* __restrict__ O, con
   float2 acc[16];
 #pragma unroll
   for (int n2 = 0; n2 < 16; ++n2) acc[n2] = make_float2(0.f, 0.f);
-  int b = next_pos(spos, before_split(split, nsplit), a.nb, nsplit);
+  int b = next_pos(a, spos, before_split(a, split, nsplit), nsplit);
   if (b >= 0) prefetch(b, 0);
   for (int buf = 0; b >= 0; buf ^= 1) {
     cp_async_wait<0>();
     __syncthreads();                                  // position b has landed; buffer buf^1 is free
-    const int bn = next_pos(spos, b, a.nb, nsplit);
+    const int bn = next_pos(a, spos, b, nsplit);
     if (bn >= 0) prefetch(bn, buf ^ 1);
     const float s = ssig[b];
     float2* reg = Sst + (buf * V + vec) * RR;
@@ -1484,7 +1488,7 @@ k_row_fwd_l(const float2* __restrict__ O, const float2* __restrict__ P, float2* 
   }
   const float2* Ol = O + a.obj_off[l];
   const int Wl = a.obj_w[l];
-  int b = next_pos(spos, before_split(split, nsplit), a.nb, nsplit);
+  int b = next_pos(a, spos, before_split(a, split, nsplit), nsplit);
   if (b >= 0) {
     prefetch_orows<F>(Ol, Wl, spos[b], row0, rpb, Ost);
     cp_async_commit();
@@ -1492,7 +1496,7 @@ k_row_fwd_l(const float2* __restrict__ O, const float2* __restrict__ P, float2* 
   for (int buf = 0; b >= 0; buf ^= 1) {
     cp_async_wait<0>();
     __syncthreads();                                  // position b's rows have landed; buf^1 is free
-    const int bn = next_pos(spos, b, a.nb, nsplit);
+    const int bn = next_pos(a, spos, b, nsplit);
     if (bn >= 0) {
       prefetch_orows<F>(Ol, Wl, spos[bn], row0, rpb, Ost + (buf ^ 1) * rpb * F);
       cp_async_commit();
@@ -1546,7 +1550,7 @@ k_row_fwd_w(const float2* __restrict__ O, const float2* __restrict__ P, float2* 
   const float2* Ol = O + a.obj_off[l];
   const int Wl = a.obj_w[l];
   const int oc = (t & 15) + 256 * (t >> 4);           // output column of x[0] (then + 16 j)
-  int b = next_pos(spos, before_split(split, nsplit), a.nb, nsplit);
+  int b = next_pos(a, spos, before_split(a, split, nsplit), nsplit);
   if (b >= 0) {
     prefetch_orows<F>(Ol, Wl, spos[b], row0, rpb, Ost);
     cp_async_commit();
@@ -1554,7 +1558,7 @@ k_row_fwd_w(const float2* __restrict__ O, const float2* __restrict__ P, float2* 
   for (int buf = 0; b >= 0; buf ^= 1) {
     cp_async_wait<0>();
     __syncthreads();                                  // position b's rows have landed; buf^1 is free
-    const int bn = next_pos(spos, b, a.nb, nsplit);
+    const int bn = next_pos(a, spos, b, nsplit);
     if (bn >= 0) {
       prefetch_orows<F>(Ol, Wl, spos[bn], row0, rpb, Ost + (buf ^ 1) * rpb * F);
       cp_async_commit();

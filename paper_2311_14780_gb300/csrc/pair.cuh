@@ -9,8 +9,8 @@
 //
 // so every load is a whole operand and no lane ever needs moving.  An odd last position has an empty
 // second lane (zeros; nothing of it is written outside the scratch).  The arithmetic of each lane is
-// that of the one-field kernels in kernels.cuh, operation by operation: the results are the same bits
-// (the probe gradient's too, given the same position splits).
+// that of the one-field kernels in kernels.cuh, operation by operation: patterns and losses are the same bits
+// given the same batches and mode groups (the probe gradient's positions are dealt to its splits in pairs here).
 //
 // Why: ncu counted 31-46 thread instructions per field element and 1D DFT in the one-field passes
 // (256^2 and 512^2), 90 ms of pure issue time in the 136 ms of the 512^2 x 6 wavelengths x 10 modes

@@ -185,6 +185,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
   a.C = p.C;
   a.MG = res ? p.MG_res : p.MG;
   a.G = res ? p.G_res : p.G;
+  a.deal = 1;
   a.status = p.d_status;
 
   LossArgs la{};

@@ -165,6 +165,7 @@ void fill_round(Site* s, int r, ptycho::SiteRound& w, int& tiles, int* counts, p
   a.chunk_len = LM;
   a.MG = p.MG;
   a.G = p.G;
+  a.deal = p.pair ? 2 : 1;                            // the order of the site's own plan
   a.status = p.d_status;
   a.patch = nullptr;
   tiles = 1;

@@ -144,3 +144,17 @@ def test_patterns_and_loss_are_the_one_field_passes_bit_by_bit(dev, F, L, M):
     assert torch.equal(*loss)
     plan.close()
     ref.close()
+
+
+def test_a_short_batch_reaches_every_split(dev):
+    """One-field passes with as many position splits as positions: every split gets one, so that the probe
+    gradient is the sum of the positions' own ones, in their order, bit by bit."""
+    case = _case(dev, 64, 1, 1, 3, 91)
+    plan = case.plan(scratch_bytes=9 * 64 * 64 * 8, flags=4)             # KEEP_PSI, the one-field default at 64^2
+    assert plan.query(PAIR_PASSES) == 0 and plan.query(ROW_ADJ_SPLITS) == plan.query(BATCH_POSITIONS) == 9
+    grad = lambda b: plan.adjoint(case.O, case.P, case.Im, case.sig_t, case.bg_t, case.mask_t, b)[2]  # noqa: E731
+    total = torch.zeros_like(case.P)
+    for j in range(9):
+        total = total + grad(torch.tensor([j], dtype=torch.int32, device=dev))
+    assert torch.equal(grad(None), total)
+    plan.close()
