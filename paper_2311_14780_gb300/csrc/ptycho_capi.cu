@@ -706,19 +706,6 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
         ns = std::min<long long>(ns, std::min<long long>(64, p->B));
         while (ns > 1 && ns * p->P_numel * (long long)sizeof(float2) > (512ll << 20)) --ns;
         p->nsplit_adj = (int)std::max<long long>(1, ns);
-        if (p->pair) {
-          // (three waves of blocks; with one mode, six warps per SM)
-          const PairSizes z = pair_sizes(F, g->M, p->rpb_pair);
-          const int ct = z.T * g->M * p->rpb_pair;
-          const long long per_sm = std::max<long long>(1, std::min<long long>(12 / (ct / 32 + ptycho::row_adj_p_feeders(ct)),
-                                                                              (220 * 1024) / (z.smem + 8 * 1024)));
-          const long long blocks = g->M == 1 ? (long long)(F * z.T / 32) * g->L : (long long)(F / p->rpb_pair) * g->L;
-          const long long want = (g->M == 1 ? 6ll : 3ll * per_sm) * p->sms;
-          long long np = (want + blocks - 1) / blocks;
-          np = std::min<long long>(np, std::min<long long>(64, (p->B + 1) / 2));
-          while (np > 1 && np * p->P_numel * (long long)sizeof(float2) > (512ll << 20)) --np;
-          p->nsplit_adj = (int)std::max<long long>(1, np);
-        }
         // the forward row pass: same blocks, positions split for four blocks per SM.  Default at
         // 512^2 from 4 modes, where the probes of all modes outgrow the L2 and the fused pass reads
         // each probe row once per block instead of once per position: measured 153.4 vs 157.2 ms
@@ -735,6 +722,27 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
         }
       }
     }
+  }
+
+  // the pair passes' row adjoint, whose block takes more modes than the one above: three waves of blocks (with
+  // one mode, six warps per SM), at most one split per pair of positions, the same bound on the buffers.
+  // Blocks of over 256 compute threads run one per SM, in whole rounds, and a split costs them a pass over their
+  // probe gradient: splits only where they save a tenth of the rounds (64^2 x 80 modes, 400 positions: 1510 us
+  // a step unsplit, 1302 with 8 splits; x 72 modes x 3 wavelengths, 200 positions: 1770 / 1666 with 3; with as
+  // many rounds either way unsplit is faster: 128^2 x 40, 100 positions: 656 / 686 with 4, 256^2 x 18: 1077 / 1092)
+  if (p->pair) {
+    const PairSizes z = pair_sizes(F, g->M, p->rpb_pair);
+    const int ct = z.T * g->M * p->rpb_pair;
+    const long long per_sm = std::max<long long>(1, std::min<long long>(12 / (ct / 32 + ptycho::row_adj_p_feeders(ct)),
+                                                                        (220 * 1024) / (z.smem + 8 * 1024)));
+    const long long blocks = g->M == 1 ? (long long)(F * z.T / 32) * g->L : (long long)(F / p->rpb_pair) * g->L;
+    const long long want = (g->M == 1 ? 6ll : 3ll * per_sm) * p->sms;
+    long long np = (want + blocks - 1) / blocks;
+    np = std::min<long long>(np, std::min<long long>(64, (p->B + 1) / 2));
+    while (np > 1 && np * p->P_numel * (long long)sizeof(float2) > (512ll << 20)) --np;
+    auto rounds = [&](long long n) { return (n * blocks + p->sms - 1) / p->sms; };
+    if (ct > 256 && 10 * rounds(np) > 9 * rounds(1) * np) np = 1;
+    p->nsplit_adj = (int)std::max<long long>(1, np);
   }
 
   // frame-resident passes (F <= 128, opt-in; measured slower than the scratch passes): all
@@ -804,7 +812,7 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
   rc = rc ? rc : dalloc(p, &p->d_gO, p->O_numel);
   rc = rc ? rc : dalloc(p, &p->d_gP, p->P_numel);
   {
-    const int ns = std::max(p->adj_l_ok ? p->nsplit_adj : 1, p->res ? p->nsplit_res : 1);
+    const int ns = std::max(p->adj_l_ok || p->pair ? p->nsplit_adj : 1, p->res ? p->nsplit_res : 1);
     if (ns > 1) rc = rc ? rc : dalloc(p, &p->d_gPs, (long long)ns * p->P_numel);
   }
   rc = rc ? rc : dalloc(p, &p->d_status, 1);

@@ -158,3 +158,16 @@ def test_a_short_batch_reaches_every_split(dev):
         total = total + grad(torch.tensor([j], dtype=torch.int32, device=dev))
     assert torch.equal(grad(None), total)
     plan.close()
+
+
+@pytest.mark.parametrize("F,L,M,splits", [(64, 1, 72, 5), (64, 3, 72, 3), (128, 1, 40, 1), (256, 1, 20, 1)])
+def test_many_modes_split_their_positions(dev, F, L, M, splits):
+    """Blocks of 288 to 320 threads run one per SM: where F L of them leave rounds half empty (64 or 192 on 152
+    SMs) the positions are split, as far as there are pairs of them (five here); 128 or 256 fill theirs as well
+    unsplit."""
+    from paper_2311_14780_gb300 import Plan
+    plan = Plan(F, L, M, 9, [(F, F)] * L, np.zeros((L, 9, 2), np.int32))
+    assert torch.cuda.get_device_properties(dev).multi_processor_count == 152
+    assert plan.query(PAIR_PASSES) == 1
+    assert plan.query(ROW_ADJ_SPLITS) == splits
+    plan.close()
