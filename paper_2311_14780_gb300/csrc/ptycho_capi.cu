@@ -527,7 +527,10 @@ int ptycho_plan_create(const ptycho_geom_t* g, ptycho_plan_t** out) {
 
 namespace ptycho {
 
-int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t** out) {
+// A plan with the given batching, with the pair passes where they apply if ``pairs``.  kNoPairMap: they would
+// apply, but the driver gave no tensor map for their scratch.
+constexpr int kNoPairMap = 1;
+static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pairs, ptycho_plan_t** out) {
   if (!g || !out) return PTYCHO_EINVAL;
   *out = nullptr;
   if (g->L < 1 || g->M < 1 || g->J < 1 || !g->obj_h || !g->obj_w || !g->pos) return PTYCHO_EINVAL;
@@ -621,7 +624,7 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
   // are the faster ones (400 positions: 3.22 vs 3.54 ms per step), at 128^2 the pair passes (246 vs 256 us;
   // at 64^2 both wait for the launches)
   constexpr int kPairFlags = PTYCHO_FLAG_NO_PDL;
-  if (p->store && !g->zoom && !(g->flags & ~kPairFlags) && p->B >= 2 && (LM >= 2 || F <= 128)) {
+  if (pairs && p->store && !g->zoom && !(g->flags & ~kPairFlags) && p->B >= 2 && (LM >= 2 || F <= 128)) {
     // rows per block of the row adjoint: whole warps of compute threads, and small blocks (64 compute
     // threads) where the modes allow it, so that several are resident and drift apart
     PairSizes z = pair_sizes(F, g->M, 1);
@@ -842,7 +845,7 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
       if (p->pair && !make_pair_map(&p->tmap_pair[i], p->d_S + (long long)i * Bs * p->C * FF, F, Bs / 2 * p->C * F,
                                     pair_sizes(F, g->M, 1).CW)) {
         free_plan(p);
-        return PTYCHO_ECUDA;
+        return kNoPairMap;
       }
     }
   }
@@ -882,6 +885,11 @@ int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t
   if (rc) { free_plan(p); return rc; }
   *out = p;
   return PTYCHO_OK;
+}
+
+int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t** out) {
+  const int rc = make_plan(g, target, true, out);
+  return rc == kNoPairMap ? make_plan(g, target, false, out) : rc;   // the one-field passes need no map
 }
 
 }  // namespace ptycho
