@@ -199,6 +199,7 @@ namespace {
 constexpr long long kMaxScratch = 8ll << 30;   // default upper bound of one buffer set
 constexpr long long kBatchElems = 320ll << 20; // field elements per batch the default aims for (1200 of 512^2)
 constexpr long long kSmallBatchElems = 8ll << 20;
+constexpr long long kBatchEvals = 1200;        // fields per batch at least, as far as the call has them
 constexpr long long kMinBatchPositions = 64;   // at least this many positions (when they fit)
 constexpr long long kMinBatches = 3;           // batches per call (overlap), when they are not small
 constexpr long long kBatchRows = 32768;        // and at least this many 1D FFT rows per pass
@@ -520,7 +521,11 @@ const char* ptycho_strerror(int code) {
 }
 
 int ptycho_plan_create(const ptycho_geom_t* g, ptycho_plan_t** out) {
-  return ptycho::create_plan(g, ptycho::BatchTarget{0, kBatchElems, kMinBatchPositions, kMaxScratch}, out);
+  // on a GPU with little memory left smaller batches, down to kBatchEvals fields (or kMinBatchPositions)
+  for (long long elems = kBatchElems;; elems /= 2) {
+    const int rc = ptycho::create_plan(g, ptycho::BatchTarget{kBatchEvals, elems, kMinBatchPositions, kMaxScratch}, out);
+    if (rc != PTYCHO_ENOMEM || g->scratch_bytes > 0 || elems <= kBatchEvals * g->F * g->F) return rc;
+  }
 }
 
 }  // extern "C"
