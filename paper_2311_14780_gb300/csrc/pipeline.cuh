@@ -367,12 +367,40 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
         PTY_LAUNCH(p, kColFwd, cs, launch_pdl(k_col_fwd<F, false>, col_grid, col_blk, ColCfg<F>::smem_xch, cs, S, Ip, a,
                                               (int)(ch == 0)));
     }
-    if (p.imeas_ready && cudaStreamWaitEvent(cs, p.imeas_ready[k], 0) != cudaSuccess) return PTYCHO_ECUDA;
-    la.npos = loss_positions(F, a.nb, p.sms);
-    PTY_LAUNCH(p, kLoss, cs, launch_pdl(k_loss<F>, dim3(loss_blocks<F>(), (a.nb + la.npos - 1) / la.npos), kLossThreads, 0,
-                                        cs, a, la));
+    // the loss and R^T, position by position: of the whole batch, or piece by piece as the measured patterns
+    // arrive (ptycho_step_host)
+    const int per = p.imeas_ready ? p.imeas_per : a.nb;
+    // (with the plain-load columns of the one-field passes also the column adjoint)
+    const bool col_plain = !pair && !p.czt && !res && !col_staged && !p.has_tma && p.nchunks == 1;
+    auto col_adj_plain = [&](float2* Sp, const KArgs& ap, const AdjArgs& ar) {
+      const dim3 grid(F / ColCfg<F>::W, p.G, ap.nb);
+      auto* kernel = F >= 512 ? (store ? k_col_adj_2b<F, true> : k_col_adj_2b<F, false>)
+                              : (store ? k_col_adj<F, true> : k_col_adj<F, false>);
+      PTY_LAUNCH(p, kColAdj, cs, launch_pdl(kernel, grid, col_blk, col_adj_smem, cs, Sp, ap, ar));
+      return (int)PTYCHO_OK;
+    };
+    const bool col_pieces = p.imeas_ready && grad && col_plain;
+    for (int i = 0, o = 0; o < a.nb; ++i, o += per) {
+      if (p.imeas_ready && cudaStreamWaitEvent(cs, p.imeas_ready[k * p.imeas_pieces + i], 0) != cudaSuccess)
+        return PTYCHO_ECUDA;
+      KArgs ap = a;
+      LossArgs lp = la;
+      AdjArgs ar = aa;
+      ap.batch_off += o;
+      ap.nb = std::min(per, a.nb - o);
+      lp.Ipart += (long long)o * a.G * FF;
+      if (lp.D) lp.D += (long long)o * FF;
+      ar.D += (long long)o * FF;
+      if (ar.Gt) ar.Gt += (long long)o * FF;
+      lp.npos = loss_positions(F, ap.nb, p.sms);
+      PTY_LAUNCH(p, kLoss, cs, launch_pdl(k_loss<F>, dim3(loss_blocks<F>(), (ap.nb + lp.npos - 1) / lp.npos), kLossThreads,
+                                          0, cs, ap, lp));
+      if (grad && p.remap)
+        PTY_LAUNCH(p, kRemapAdj, cs, launch_pdl(k_remap_adj<F>, dim3(FF / 256, (ap.nb + kRtPos - 1) / kRtPos), 256, 0, cs,
+                                                ap, ar));
+      if (col_pieces && (rc = col_adj_plain(S + (long long)o * p.C * FF, ap, ar)) != PTYCHO_OK) return rc;
+    }
     if (!grad) continue;
-    if (p.remap) PTY_LAUNCH(p, kRemapAdj, cs, launch_pdl(k_remap_adj<F>, dim3(FF / 256, (a.nb + kRtPos - 1) / kRtPos), 256, 0, cs, a, aa));
     if (c.g_bg)                                       // per-set background-gradient sum, batch order
       PTY_LAUNCH(p, kRemapAdj, cs, launch_pdl(k_bg_accum<F>, dim3(FF / 256), 256, 0, cs,
                                               (const float*)(p.remap ? aa.Gt : aa.D), a.nb, p.d_gbg_set + set * FF));
@@ -417,7 +445,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
       if (!store && rerun_rows)
         PTY_LAUNCH(p, kRowFwd, cs,
                    launch_pdl(k_row_fwd<F>, dim3(a.nb, F / RowCfg<F>::RPB, p.L), row_blk, RowCfg<F>::smem, cs, c.O, c.P, S, a));
-      if (pair)
+      if (pair || col_pieces)
         ;
       else if (col_staged) {
         rc = narrow ? launch_cols_s<F, 4>(p, false, store, cs, S, Ip, a, aa) : launch_cols_s<F, 0>(p, false, store, cs, S, Ip, a, aa);
@@ -432,14 +460,8 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
       else if (p.has_tma)
         PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_col_adj_tma<F, false>, col_grid, col_blk, ColTma<F>::smem_adj, cs,
                                               p.tmap_S[set], S, a, aa));
-      else if (F >= 512 && store)
-        PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_col_adj_2b<F, true>, col_grid, col_blk, col_adj_smem, cs, S, a, aa));
-      else if (F >= 512)
-        PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_col_adj_2b<F, false>, col_grid, col_blk, col_adj_smem, cs, S, a, aa));
-      else if (store)
-        PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_col_adj<F, true>, col_grid, col_blk, col_adj_smem, cs, S, a, aa));
-      else
-        PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_col_adj<F, false>, col_grid, col_blk, col_adj_smem, cs, S, a, aa));
+      else if ((rc = col_adj_plain(S, a, aa)) != PTYCHO_OK)
+        return rc;
       // the probe and object gradients accumulate in batch order across the streams
       if (nsets > 1 && k > 0 && cudaStreamWaitEvent(cs, p.ev_radj[(k - 1) % nsets], 0) != cudaSuccess)
         return PTYCHO_ECUDA;

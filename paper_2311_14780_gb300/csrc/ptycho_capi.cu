@@ -204,6 +204,9 @@ constexpr long long kMinBatchPositions = 64;   // at least this many positions (
 constexpr long long kMinBatches = 3;           // batches per call (overlap), when they are not small
 constexpr long long kBatchRows = 32768;        // and at least this many 1D FFT rows per pass
 constexpr int kDefaultOverlap = 3;             // position batches in flight
+constexpr long long kHostPieceBytes = 6 << 20; // ptycho_step_host: measured patterns per copy at least,
+constexpr int kHostPieces = 4;                 // copies per call at most where it has few batches,
+constexpr int kHostPieceFields = 4;            // and in pieces for plans of fewer fields per position
 constexpr double kPi = 3.14159265358979323846;
 
 bool supported_F(int F) { return F == 64 || F == 128 || F == 256 || F == 512; }
@@ -1170,15 +1173,26 @@ int ptycho_step_host(ptycho_plan_t* p, ptycho_adam_t* s, float* O, float* P, flo
     }
     rc = ptycho_step(p, s, O, P, sigma, bg, I_meas_dev, mask, mask_per_frame, batch_idx, nbatch, loss_dev, stream);
   } else {
-    // all positions in order: batch k's frames are copied on a side stream after the work queued
-    // on stream so far, and its loss kernel waits only for them, so the copies of later batches
-    // overlap the transforms of earlier ones
+    // all positions in order: the frames are copied on a side stream after the work queued on stream so
+    // far, and a batch's loss kernels wait only for theirs, so the copies of later batches overlap the
+    // transforms of earlier ones.  A call of one or two batches has little to overlap a copy with but its
+    // forward passes, and those are shorter than the copy up to about four fields per position (copy 19 ps,
+    // forward 5 ps per pixel and field): there a batch comes in pieces, and the passes that work position by
+    // position on what has arrived (loss, R^T, plain-load columns) overlap the next piece's copy.  us per
+    // call, one copy / pieces (three batches): 512^2, one field, 60 positions 715 / 581 (613); 128^2, 400: 320 /
+    // 294 (293); 256^2, 100: 317 / 287 (282); 256^2, two fields, 60: 229 / 217 (229)
     if (!p->copy_st && (cudaStreamCreateWithFlags(&p->copy_st, cudaStreamNonBlocking) != cudaSuccess ||
                         cudaEventCreateWithFlags(&p->ev_copy_start, cudaEventDisableTiming) != cudaSuccess)) {
       cudaGetLastError();
       return PTYCHO_ECUDA;
     }
-    while ((int)p->ev_copy.size() < nbat) {
+    const long long whole = (long long)(frame * (size_t)p->B) / kHostPieceBytes;
+    const int want = p->L * p->M < kHostPieceFields
+                         ? (int)std::max<long long>(1, std::min<long long>(nbat < kMinBatches ? kHostPieces / nbat : 1, whole))
+                         : 1;
+    p->imeas_per = ((p->B + want - 1) / want + 7) / 8 * 8;            // whole groups of the loss pass and of R^T
+    p->imeas_pieces = (p->B + p->imeas_per - 1) / p->imeas_per;
+    while ((int)p->ev_copy.size() < nbat * p->imeas_pieces) {
       cudaEvent_t e;
       if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return PTYCHO_ECUDA;
       p->ev_copy.push_back(e);
@@ -1187,13 +1201,16 @@ int ptycho_step_host(ptycho_plan_t* p, ptycho_adam_t* s, float* O, float* P, flo
         cudaStreamWaitEvent(p->copy_st, p->ev_copy_start, 0) != cudaSuccess)
       return PTYCHO_ECUDA;
     for (int k = 0; k < nbat; ++k) {
-      const size_t off = (size_t)k * p->B, n = (size_t)std::min(p->B, p->J - k * p->B);
-      if (cudaMemcpyAsync(reinterpret_cast<char*>(I_meas_dev) + off * frame,
-                          reinterpret_cast<const char*>(I_meas_host) + off * frame, n * frame,
-                          cudaMemcpyHostToDevice, p->copy_st) != cudaSuccess ||
-          cudaEventRecord(p->ev_copy[k], p->copy_st) != cudaSuccess) {
-        cudaGetLastError();
-        return PTYCHO_ECUDA;
+      const int nb = std::min(p->B, p->J - k * p->B);
+      for (int i = 0, o = 0; o < nb; ++i, o += p->imeas_per) {
+        const size_t off = (size_t)k * p->B + o, n = (size_t)std::min(p->imeas_per, nb - o);
+        if (cudaMemcpyAsync(reinterpret_cast<char*>(I_meas_dev) + off * frame,
+                            reinterpret_cast<const char*>(I_meas_host) + off * frame, n * frame,
+                            cudaMemcpyHostToDevice, p->copy_st) != cudaSuccess ||
+            cudaEventRecord(p->ev_copy[k * p->imeas_pieces + i], p->copy_st) != cudaSuccess) {
+          cudaGetLastError();
+          return PTYCHO_ECUDA;
+        }
       }
     }
     p->imeas_ready = p->ev_copy.data();
