@@ -78,6 +78,13 @@ __device__ __forceinline__ cpair cscale(cpair a, float2 s) {
           make_float2(__fmul_rn(a.im.x, s.x), __fmul_rn(a.im.y, s.y))};
 }
 
+// acc += |v|^2 with one rounding of the sum, which grows over the modes, and not one for each part of v:
+// with 40 modes in one sum (128^2 x 8 x 5) the object gradient's error was 2.7 % above that of two sums of 20.
+__device__ __forceinline__ void add_abs2(float& acc, float2 v) { acc = __fadd_rn(acc, fmaf(v.x, v.x, __fmul_rn(v.y, v.y))); }
+__device__ __forceinline__ void add_abs2(float2& acc, cpair v) {
+  acc = __fadd2_rn(acc, __ffma2_rn(v.re, v.re, __fmul2_rn(v.im, v.im)));
+}
+
 // cos(2*pi*i/32) for i in [0, 8]
 __host__ __device__ constexpr double kCos32(int i) {
   return i == 0 ? 1.0

@@ -207,7 +207,7 @@ __device__ __forceinline__ void col_fwd_body(float2* __restrict__ S, float* __re
     fft_fwd_I2O<F>(v, t, smem + c * Xch<F>::region_cols, a.tw, BlockSync{});
 #pragma unroll
     for (int sl = 0; sl < N2; ++sl) {
-      acc[sl] = fmaf(v[sl].x, v[sl].x, fmaf(v[sl].y, v[sl].y, acc[sl]));
+      add_abs2(acc[sl], v[sl]);
       if (STORE) base[(long long)idxO<F>(t, sl) * F] = cscale(v[sl], inv);
     }
   }
@@ -304,7 +304,7 @@ k_col_fwd_tma(const __grid_constant__ CUtensorMap map, float2* __restrict__ S, f
     float2* base = S + ((long long)b * a.C + cm) * F * F + col;
 #pragma unroll
     for (int sl = 0; sl < N2; ++sl) {
-      acc[sl] = fmaf(v[sl].x, v[sl].x, fmaf(v[sl].y, v[sl].y, acc[sl]));
+      add_abs2(acc[sl], v[sl]);
       if (STORE) base[(long long)idxO<F>(t, sl) * F] = cscale(v[sl], inv);
     }
   }
@@ -391,7 +391,7 @@ k_col_fwd_s(float2* __restrict__ S, float* __restrict__ Ipart, KArgs a) {
     float2* base = Sb + (long long)cm * F * F + col;
 #pragma unroll
     for (int sl = 0; sl < N2; ++sl) {
-      acc[sl] = fmaf(v[sl].x, v[sl].x, fmaf(v[sl].y, v[sl].y, acc[sl]));
+      add_abs2(acc[sl], v[sl]);
       if (STORE) base[(long long)idxO<F>(t, sl) * F] = cscale(v[sl], inv);
     }
   }
@@ -981,7 +981,7 @@ k_col_fwd_tma2(const __grid_constant__ CUtensorMap map, float* __restrict__ Ipar
     if (threadIdx.x == 0 && cm + 1 < m1) col_tma_issue<F>(stage, &map, col0, ((long long)b * a.C + cm + 1) * F, bar);
     fft_fwd_I2O_half<F>(v, t, xch + c * R, a.tw, BlockSync{});
 #pragma unroll
-    for (int sl = 0; sl < N2; ++sl) acc[sl] = fmaf(v[sl].x, v[sl].x, fmaf(v[sl].y, v[sl].y, acc[sl]));
+    for (int sl = 0; sl < N2; ++sl) add_abs2(acc[sl], v[sl]);
   }
   if (!ok) {                                   // give a lost copy a bounded chance to land, then stop
     if (threadIdx.x == 0) mbar_wait_bounded(bar, phase, a.status);

@@ -467,7 +467,7 @@ k_col_fwd_p(const __grid_constant__ CUtensorMap map, float* __restrict__ Ipart, 
     for (int i = 0; i < 16; ++i) x[i] = ld_pair(pl.elem(i));
     pair_fwd<F>(x, t, pl, tw);
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = __ffma2_rn(x[i].re, x[i].re, __ffma2_rn(x[i].im, x[i].im, acc[i]));
+    for (int i = 0; i < 16; ++i) add_abs2(acc[i], x[i]);
   }
   if (!ok) {                                          // give a lost copy a bounded chance to land, then stop
     if (threadIdx.x == 0) mbar_wait_bounded(&bar[k & 1], (k >> 1) & 1, a.status);

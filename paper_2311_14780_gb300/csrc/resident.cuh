@@ -108,7 +108,7 @@ k_res_fwd(const float2* __restrict__ O, const float2* __restrict__ P, float* __r
         for (int n2 = 0; n2 < N2; ++n2) z[n2] = fr[(t + N1 * n2) * C::pitch + c];
         fft_fwd_I2O<F>(z, t, xc, a.tw, WarpSync{});
 #pragma unroll
-        for (int sl = 0; sl < N2; ++sl) acc[rho][sl] = fmaf(z[sl].x, z[sl].x, fmaf(z[sl].y, z[sl].y, acc[rho][sl]));
+        for (int sl = 0; sl < N2; ++sl) add_abs2(acc[rho][sl], z[sl]);
       }
       __syncthreads();                                // the frame is rewritten by the next mode
     }

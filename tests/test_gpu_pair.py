@@ -171,3 +171,23 @@ def test_many_modes_split_their_positions(dev, F, L, M, splits):
     assert plan.query(PAIR_PASSES) == 1
     assert plan.query(ROW_ADJ_SPLITS) == splits
     plan.close()
+
+
+# the pair and the one-field column passes (plain, TMA, staged, recomputed, one block per SM, without TMA)
+@pytest.mark.parametrize("F,M,flags", [(64, 40, 0), (64, 40, 4), (64, 40, 16), (64, 40, 64), (128, 40, 0), (128, 8, 4),
+                                       (256, 20, 0), (256, 20, 1), (512, 10, 0), (512, 10, 1), (512, 10, 65536),
+                                       (512, 10, 8), (512, 10, 4), (512, 10, 64)])
+def test_intensity_sum_rounds_once_per_mode(dev, F, M, flags):
+    """Constant objects and probes put all of a mode into the pattern's centre, exactly: |Psi_m|^2 = F^2 |c_m|^2.
+    The first mode's 2^24 has a unit of 2 in its last place, so each later one may cost half of it, 1; adding
+    the squares of the real and the imaginary part (0.77 each) one after the other would lose both."""
+    from paper_2311_14780_gb300 import Plan
+    plan = Plan(F, 1, M, 2, [(F, F)], np.zeros((1, 2, 2), np.int32), flags=flags, col_groups=1)
+    assert plan.query(COLUMN_GROUPS) == 1
+    c = torch.full((1, M, 1, 1), 0.875 + 0.875j, dtype=torch.complex64, device=dev)
+    c[0, 0] = 4096.0
+    I = plan.forward(torch.ones(F * F, dtype=torch.complex64, device=dev), c.expand(1, M, F, F).contiguous())
+    centre = I[:, F // 2, F // 2].double().cpu().numpy() / F ** 2
+    assert np.abs(centre - (2.0 ** 24 + (M - 1) * 1.53125)).max() <= M - 1
+    assert float(I.double().sum().item()) == float(I[:, F // 2, F // 2].double().sum().item())
+    plan.close()
