@@ -54,8 +54,9 @@ extern "C" {
  * Without a flag (or with NO_PDL alone) a plan that keeps all modes of a position in the scratch, with
  * at least two positions per batch and two fields per position (one at F <= 128), transforms pairs of
  * positions in the packed FP32 lanes (csrc/pair.cuh), where its row adjoint's block fits (any
- * count up to 10 modes; up to 20, 40 and 72 at F = 256, 128 and 64 where the count fills whole warps in
- * a block of at most 320 threads).  Any other flag selects the one-field passes, whose variants and defaults the following describes.
+ * count up to 10 modes; up to 20, 40 and 80 at F = 256, 128 and 64 where the count fills whole warps in
+ * a block of at most 320 threads).  Any other flag selects the one-field passes, whose variants and
+ * defaults the following describes.  PTYCHO_QUERY_PAIR_PASSES says which a plan took.
  * RECOMPUTE_COLUMNS: the adjoint recomputes the column DFT from the kept row-pass output
  *   instead of keeping Psi (less memory traffic, one more 1D pass per evaluation); the
  *   default for F >= 256, where it measured faster.
@@ -158,10 +159,13 @@ typedef struct {
   int32_t remap;            /* 1: apply the tilted-plane remap inside f5; 0: identity   */
   int32_t loss;             /* PTYCHO_LOSS_AMPLITUDE, _POISSON or _POISSON_GAUSSIAN     */
   float eps;                /* intensity floor added to I in the loss and its gradient  */
-  int64_t scratch_bytes;    /* FFT scratch budget in bytes; 0 = library default (about
-                               1200 evaluations but at least 64 positions per batch, at
-                               least three batches per call, batches of equal size within
-                               one position, at most 8 GiB per buffer set)              */
+  int64_t scratch_bytes;    /* FFT scratch budget in bytes; 0 = library default: 320 Mi
+                               field elements per batch (2.5 GB; L M F^2 of them per
+                               position) but at least 64 positions and at most 512 or
+                               8 GiB; three batches per call where each holds 8 Mi elements
+                               (2 Mi with zoom), else two or one; of equal size within one
+                               position (two with the pair passes).  On PTYCHO_ENOMEM the
+                               target is halved, down to 1200 fields or 64 positions.    */
   int32_t overlap;          /* position batches in flight on separate streams (1..4), each
                                with its own scratch set; 0 = library default (3)       */
   int32_t flags;            /* PTYCHO_FLAG_* variants; 0 = defaults                      */
@@ -372,8 +376,8 @@ int64_t ptycho_plan_query(const ptycho_plan_t* plan, int what);
 
 /* Device-side status of the plan since the previous query, then cleared.  Bit 0
  * (PTYCHO_STATUS_BAD_INDEX): a batch_idx entry was outside [0, J); that position was
- * skipped.  Bit 1 (PTYCHO_STATUS_WAIT_TIMEOUT): a bulk shared-memory copy of a column pass
- * did not complete within about a second; the block gave up and its outputs for that call
+ * skipped.  Bit 1 (PTYCHO_STATUS_WAIT_TIMEOUT): a bulk shared-memory copy of a row or column
+ * pass did not complete within about a second; the block gave up and its outputs for that call
  * are not valid.  Synchronises the device (call it outside the timed loop). */
 #define PTYCHO_STATUS_BAD_INDEX 1
 #define PTYCHO_STATUS_WAIT_TIMEOUT 2

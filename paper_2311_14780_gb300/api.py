@@ -178,7 +178,7 @@ class Plan:
 
     def status(self) -> int:
         """Device status flags since the last query (synchronises; bit 0 = bad batch index,
-        bit 1 = a column pass's bulk copy timed out)."""
+        bit 1 = a row or column pass's bulk copy timed out)."""
         v = ctypes.c_int32(0)
         _check(_native.lib().ptycho_plan_status(self._h_plan, ctypes.byref(v)), "ptycho_plan_status")
         return int(v.value)

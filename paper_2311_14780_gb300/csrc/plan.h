@@ -173,8 +173,8 @@ struct BatchTarget {
 int create_plan(const ptycho_geom_t* g, const BatchTarget& target, ptycho_plan_t** out);
 // Evaluations per position batch of a served site, in both tick forms.  Measured on the
 // 64-request serving stream: per-site graphs 576 / 649 / 659 K evals/s with 128 / 600 / 1200;
-// shared launches 468 / 500 / 519 / 524 K with 300 / 600 / 1200 / 2400.  1200 is also the
-// single-site default, so a site's scratch is what its own plan would take.
+// shared launches 468 / 500 / 519 / 524 K with 300 / 600 / 1200 / 2400.  A plan of its own would take
+// more on small frames (kBatchElems); many sites share the GPU's memory here, and their passes overlap.
 constexpr long long kServeBatchEvals = 1200;
 constexpr BatchTarget kServeBatchTarget{kServeBatchEvals, 0, 1, 2ll << 30};
 

@@ -197,7 +197,7 @@ namespace {
 // element counts for four (two transforms of 2 F points per axis, bound by arithmetic: short batches lose
 // little and their overlap fills the tails): 64^2 x 5 x 2 with 151 / 51 of 151 positions 556 / 507 us.
 constexpr long long kMaxScratch = 8ll << 30;   // default upper bound of one buffer set
-constexpr long long kBatchElems = 320ll << 20; // field elements per batch the default aims for (1200 of 512^2)
+constexpr long long kBatchElems = 320ll << 20; // field elements per batch the default aims for (1280 of 512^2)
 constexpr long long kSmallBatchElems = 8ll << 20;
 constexpr long long kBatchEvals = 1200;        // fields per batch at least, as far as the call has them
 constexpr long long kMinBatchPositions = 64;   // at least this many positions (when they fit)
@@ -629,8 +629,12 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
   }
   // passes over pairs of positions, unless a variant flag asks for the one-field passes.  With one field
   // per position a column tile has no second mode to fetch meanwhile: at 512^2 the one-field column passes
-  // are the faster ones (400 positions: 3.22 vs 3.54 ms per step), at 128^2 the pair passes (246 vs 256 us;
-  // at 64^2 both wait for the launches)
+  // are the faster ones (us per step, pair / one-field: 60 positions 533 / 497, 400: 2860 / 2598), at 256^2 both
+  // are even on short calls (25: 85 / 84, 100: 216 / 217; 400: 681 / 704), at 128^2 the pair passes (100: 87 /
+  // 94, 400: 225 / 236; 64^2: 108 / 121 with 400, else waiting for the launches).
+  // One mode and several wavelengths: the pair passes from two fields on (us per step, pair / one-field:
+  // 512^2 x 2 wavelengths x 400 positions 4006 / 4136, x 3 x 200 2813 / 2907, x 6 x 100 2396 / 2676;
+  // 256^2 x 2 x 200 520 / 580, x 3 x 300 938 / 1167; 128^2 x 2 x 200 183 / 207)
   constexpr int kPairFlags = PTYCHO_FLAG_NO_PDL;
   if (pairs && p->store && !g->zoom && !(g->flags & ~kPairFlags) && p->B >= 2 && (LM >= 2 || F <= 128)) {
     // rows per block of the row adjoint: whole warps of compute threads, and small blocks (64 compute
