@@ -162,10 +162,12 @@ typedef struct {
   int64_t scratch_bytes;    /* FFT scratch budget in bytes; 0 = library default: 320 Mi
                                field elements per batch (2.5 GB; L M F^2 of them per
                                position) but at least 64 positions and at most 512 or
-                               8 GiB; three batches per call where each holds 8 Mi elements
-                               (2 Mi with zoom), else two or one; of equal size within one
-                               position (two with the pair passes).  On PTYCHO_ENOMEM the
-                               target is halved, down to 1200 fields or 64 positions.    */
+                               8 GiB; three batches per call where each holds 8 Mi elements,
+                               else two or one; of equal size within one position (two with
+                               the pair passes).  With zoom 1200 fields per batch, and three
+                               batches per call or, below 4 Mi elements and 8 + 4096 / F
+                               positions, one.  On PTYCHO_ENOMEM the target is halved, down
+                               to 1200 fields or 64 positions.                           */
   int32_t overlap;          /* position batches in flight on separate streams (1..4), each
                                with its own scratch set; 0 = library default (3)       */
   int32_t flags;            /* PTYCHO_FLAG_* variants; 0 = defaults                      */

@@ -193,9 +193,13 @@ namespace {
 // 256^2 x 4 x 3 with 50 / 68 / 100 / 134 3.18 / 3.13 / 3.06 / 3.00 ms: so the target is in elements.
 // One field per position: 64^2 with 22 / 32 / 64 of 64 positions 139 / 117 / 98 us (launches), 128^2
 // with 68 / 134 / 200 / 400 of 400 positions 262 / 243 / 235 / 241 us; 256^2 x 6 modes x 2 wavelengths
-// with 10 / 13 of 25 positions 311 / 283 us.  So batches of under kSmallBatchElems are merged.  A chirp-z
-// element counts for four (two transforms of 2 F points per axis, bound by arithmetic: short batches lose
-// little and their overlap fills the tails): 64^2 x 5 x 2 with 151 / 51 of 151 positions 556 / 507 us.
+// with 10 / 13 of 25 positions 311 / 283 us.  So batches of under kSmallBatchElems are merged.
+// Chirp-z passes: the per-mode row adjoint takes a batch's positions one after another in few blocks, a chain that
+// overlapping batches hide and that grows with the batch.  So they keep batches of kBatchEvals fields (64^2 x 4 x
+// 2 with 128 / 256 of 768 positions 1937 / 2119 us a step), and calls of under kSmallBatchElems / 2 are merged only
+// below 8 + 4096 / F positions (us a step in one batch / three: 64^2 x 5 fields 26 positions 119 / 131, 51 189 /
+// 187, 102 335 / 310; 128^2 x 8: 16 130 / 172, 48 314 / 302; 256^2 x 1: 16 108 / 117, 32 170 / 171, 48 235 / 227;
+// with more elements 128^2 x 30, 26 positions: 669 / 559).
 constexpr long long kMaxScratch = 8ll << 30;   // default upper bound of one buffer set
 constexpr long long kBatchElems = 320ll << 20; // field elements per batch the default aims for (1280 of 512^2)
 constexpr long long kSmallBatchElems = 8ll << 20;
@@ -608,11 +612,12 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
     long long B = p->scratch_budget / (LM * FF8);
     if (g->scratch_bytes <= 0) {
       const long long elems = LM * F * F;               // of one position
-      const long long evals = std::max(target.evals, (target.elems + F * F - 1) / (F * F));
+      const long long evals = g->zoom ? kBatchEvals : std::max(target.evals, (target.elems + F * F - 1) / (F * F));
       B = std::min<long long>(B, std::max({(evals + LM - 1) / LM, (kBatchRows + LM * F - 1) / (LM * F),
                                            target.min_positions}));
-      const long long work = g->J * elems * (g->zoom ? 4 : 1);
-      const long long nmin = std::max<long long>(1, std::min<long long>(kMinBatches, work / kSmallBatchElems));
+      const long long whole = !g->zoom ? g->J * elems / kSmallBatchElems
+                              : g->J * elems < kSmallBatchElems / 2 && g->J < 8 + 4096 / F ? 1 : kMinBatches;
+      const long long nmin = std::max<long long>(1, std::min<long long>(kMinBatches, whole));
       B = std::min<long long>(B, std::max<long long>(1, (g->J + nmin - 1) / nmin));
     }
     p->B = (int)std::max<long long>(1, std::min<long long>(B, ptycho::kMaxB));

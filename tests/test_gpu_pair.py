@@ -191,3 +191,14 @@ def test_intensity_sum_rounds_once_per_mode(dev, F, M, flags):
     assert np.abs(centre - (2.0 ** 24 + (M - 1) * 1.53125)).max() <= M - 1
     assert float(I.double().sum().item()) == float(I[:, F // 2, F // 2].double().sum().item())
     plan.close()
+
+
+@pytest.mark.parametrize("F,fields,J,batch", [(64, 5, 71, 71), (64, 5, 72, 24), (128, 8, 31, 31), (128, 8, 32, 11), (128, 30, 26, 9),
+                                              (64, 8, 768, 128), (512, 1, 15, 15), (512, 1, 16, 6)])
+def test_chirp_z_batches(dev, F, fields, J, batch):
+    """Chirp-z batches hold 1200 fields (and at least 64 positions); a call is one batch instead of three only with few
+    positions and few elements."""
+    from paper_2311_14780_gb300 import Plan
+    plan = Plan(F, 1, fields, J, [(F, F)], np.zeros((1, J, 2), np.int32), zoom=[1.0])
+    assert plan.query(BATCH_POSITIONS) == batch
+    plan.close()
