@@ -746,10 +746,12 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
 
   // the pair passes' row adjoint, whose block takes more modes than the one above: three waves of blocks (with
   // one mode, six warps per SM), at most one split per pair of positions, the same bound on the buffers.
-  // Blocks of over 256 compute threads run one per SM, in whole rounds, and a split costs them a pass over their
-  // probe gradient: splits only where they save a tenth of the rounds (64^2 x 80 modes, 400 positions: 1510 us
-  // a step unsplit, 1302 with 8 splits; x 72 modes x 3 wavelengths, 200 positions: 1770 / 1666 with 3; with as
-  // many rounds either way unsplit is faster: 128^2 x 40, 100 positions: 656 / 686 with 4, 256^2 x 18: 1077 / 1092)
+  // Blocks run in whole rounds, and a split costs a pass over the probe gradient: blocks of over 256 compute threads
+  // (one per SM) and those of several rounds are split only where that saves a tenth of the rounds (64^2 x 80
+  // modes, 400 positions: 1510 us a step unsplit, 1302 with 8 splits; x 72 modes x 3 wavelengths, 200 positions: 1770 /
+  // 1666 with 3; with as many rounds either way unsplit is faster: 128^2 x 40, 100 positions: 656 / 686 with 4, 256^2 x
+  // 10 x 3, 9 positions: 300 / 329 with 2).  Smaller blocks of one round gain from splits all the same, their tails
+  // overlap (256^2 x 3 x 2, 61 positions: 382 / 355 with 4)
   if (p->pair) {
     const PairSizes z = pair_sizes(F, g->M, p->rpb_pair);
     const int ct = z.T * g->M * p->rpb_pair;
@@ -760,8 +762,9 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
     long long np = (want + blocks - 1) / blocks;
     np = std::min<long long>(np, std::min<long long>(64, (p->B + 1) / 2));
     while (np > 1 && np * p->P_numel * (long long)sizeof(float2) > (512ll << 20)) --np;
-    auto rounds = [&](long long n) { return (n * blocks + p->sms - 1) / p->sms; };
-    if (ct > 256 && 10 * rounds(np) > 9 * rounds(1) * np) np = 1;
+    const long long slots = per_sm * p->sms;
+    auto rounds = [&](long long n) { return (n * blocks + slots - 1) / slots; };
+    if (g->M > 1 && (ct > 256 || rounds(1) > 1) && 10 * rounds(np) > 9 * rounds(1) * np) np = 1;
     p->nsplit_adj = (int)std::max<long long>(1, np);
   }
 

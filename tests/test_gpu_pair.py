@@ -202,3 +202,14 @@ def test_chirp_z_batches(dev, F, fields, J, batch):
     plan = Plan(F, 1, fields, J, [(F, F)], np.zeros((1, J, 2), np.int32), zoom=[1.0])
     assert plan.query(BATCH_POSITIONS) == batch
     plan.close()
+
+
+@pytest.mark.parametrize("F,L,M,J,splits", [(256, 3, 10, 9, 1), (256, 2, 3, 60, 4), (256, 3, 4, 60, 3), (128, 5, 8, 60, 3)])
+def test_splits_follow_the_rounds_of_blocks(dev, F, L, M, J, splits):
+    """Several rounds of blocks are split where that saves a tenth of them (768 blocks of 10 modes on 304 places: three
+    rounds either way), one round always (256 blocks of three modes)."""
+    from paper_2311_14780_gb300 import Plan
+    plan = Plan(F, L, M, J, [(F, F)] * L, np.zeros((L, J, 2), np.int32))
+    assert torch.cuda.get_device_properties(dev).multi_processor_count == 152
+    assert plan.query(ROW_ADJ_SPLITS) == splits
+    plan.close()
