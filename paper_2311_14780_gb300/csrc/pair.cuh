@@ -309,6 +309,12 @@ __device__ __forceinline__ PairPos pair_pos(const KArgs& a, int p, int l) {
 // rows in L2; a block takes about kRowFwdPairs pairs, so that the rows in use stay far below its size.
 // ---------------------------------------------------------------------------------------
 constexpr int kRowFwdPairs = 4;
+// Calls of a pair plan that take the one-field passes: subsets of up to this many positions, whose pairs are too few
+// blocks for the chip (a single position leaves half of every pass empty as well).  us a step, pair / one-field:
+// 256^2 x 30 fields 3 positions 198 / 161, 6 218 / 214, 8 257 / 270; 256^2 x 10 5 117 / 100, 9 148 / 131, 12 156 / 159;
+// 256^2 x 8 3 84 / 76, 7 114 / 104, 11 134 / 135; 128^2 x 30 3 98 / 89, 9 123 / 110, 12 138 / 131; 64^2 x 30 4 82 / 79,
+// 12 83 / 87; 512^2 x 8 4 225 / 240.
+constexpr int pair_subset(int F) { return F == 512 ? 1 : F == 128 ? 16 : 10; }
 
 template <int F, bool BULK>
 __global__ void __launch_bounds__(128, 3)

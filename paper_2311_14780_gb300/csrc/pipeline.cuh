@@ -163,7 +163,9 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
   // mode-summed object-gradient patch that the adjoint shift transforms)
   const bool shifted = p.d_delta != nullptr;
   if (shifted && (p.nchunks != 1 || !p.adj_l_ok)) return PTYCHO_EUNSUPPORTED;
-  const bool pair = p.pair != 0;                      // passes over pairs of positions
+  // passes over pairs of positions, but for small calls (pair_subset)
+  const int nb1 = c.nbatch < p.B ? c.nbatch : p.B;    // positions of the largest batch
+  const bool pair = p.pair != 0 && !(c.nbatch < p.J && nb1 <= pair_subset(F));
   const bool adj_l = (p.adj_l && !obj_atomic && p.nchunks == 1) || shifted || pair;
   const bool col_staged = p.col_staged && p.nchunks == 1;
   const bool fwd_l = p.fwd_l && p.nchunks == 1 && !shifted;
@@ -171,7 +173,11 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
   // frame-resident passes (F <= 128, PTYCHO_FLAG_RESIDENT_FRAMES): fields stay in one block's
   // shared memory
   const bool res = ResSupported<F>::value && p.res && !shifted && !p.czt && p.nchunks == 1 && !obj_atomic;
-  const int nsplit = res ? p.nsplit_res : adj_l ? p.nsplit_adj : 1;
+  // (splits without a position would only be cleared and added)
+  const int nsplit = res     ? p.nsplit_res
+                     : !adj_l ? 1
+                     : pair   ? std::min(p.nsplit_adj, (nb1 + 1) / 2)
+                              : std::min(p.pair ? p.nsplit_one : p.nsplit_adj, nb1);
   float2* gPs = nsplit > 1 ? p.d_gPs : c.gP;
 
   KArgs a{};
@@ -183,8 +189,10 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
   a.sigma = c.sigma;
   a.tw = p.d_tw;
   a.C = p.C;
-  a.MG = res ? p.MG_res : p.MG;
-  a.G = res ? p.G_res : p.G;
+  const bool few = p.G_few > 0 && 2 * nb1 <= p.B;
+  a.MG = res ? p.MG_res : few ? p.MG_few : p.MG;
+  a.G = res ? p.G_res : few ? p.G_few : p.G;
+  if (p.pair && !pair) a.G = small_call_groups(p, F / ColCfg<F>::W, nb1, a.MG);
   a.deal = 1;
   a.status = p.d_status;
 
@@ -232,7 +240,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
   const int col_adj_smem = ColCfg<F>::smem_xch + F * ColCfg<F>::W * (int)sizeof(float);
   const int nbatches = (c.nbatch + p.B - 1) / p.B;
   const int nsets = p.nsets < nbatches ? p.nsets : nbatches;
-  const long long set_S = (long long)(pair ? (p.B + 1) / 2 * 2 : p.B) * p.C * FF, set_I = (long long)p.B * a.G * FF, set_F = (long long)p.B * FF;
+  const long long set_S = (long long)(p.pair ? (p.B + 1) / 2 * 2 : p.B) * p.C * FF, set_I = p.Ipart_slices * FF, set_F = (long long)p.B * FF;
   cudaStream_t streams[ptycho_plan::kMaxSets] = {st};
   for (int i = 1; i < nsets; ++i) streams[i] = p.side[i - 1];
   if (nsets > 1) {                                    // the side streams follow the caller's work so far
@@ -304,7 +312,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
         if (p.czt) {                                  // chirp-z propagator
           PTY_LAUNCH(p, kRowFwd, cs, launch_pdl(k_czt_row_fwd<F>, dim3(a.nb, F / CztRowCfg<F>::RPB, p.L),
                                                 CztRowCfg<F>::threads, CztRowCfg<F>::smem, cs, c.O, c.P, S, a, ct));
-          PTY_LAUNCH(p, kColFwd, cs, launch_pdl(k_czt_col_fwd<F>, dim3(F / CztColCfg<F>::W, p.G, a.nb),
+          PTY_LAUNCH(p, kColFwd, cs, launch_pdl(k_czt_col_fwd<F>, dim3(F / CztColCfg<F>::W, a.G, a.nb),
                                                 CztColCfg<F>::threads, CztColCfg<F>::smem_fwd, cs, (const float2*)S, Ip,
                                                 a, ct));
           continue;
@@ -318,7 +326,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
         const int chunks = std::min(np, std::max(want, (np + kRowFwdPairs - 1) / kRowFwdPairs));
         PTY_LAUNCH(p, kRowFwd, cs, launch_pdl(k_fwd, dim3(chunks, rows, p.L), 128, PairCfg<F>::smem_row_fwd, cs, c.O, c.P,
                                               reinterpret_cast<float4*>(S), a));
-        PTY_LAUNCH(p, kColFwd, cs, launch_pdl(k_col_fwd_p<F>, dim3(F / PairCfg<F>::CW, p.G, np), PairCfg<F>::cthreads,
+        PTY_LAUNCH(p, kColFwd, cs, launch_pdl(k_col_fwd_p<F>, dim3(F / PairCfg<F>::CW, a.G, np), PairCfg<F>::cthreads,
                                               PairCfg<F>::smem_col, cs, p.tmap_pair[set], Ip, a));
         continue;
       }
@@ -340,7 +348,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
       else
         PTY_LAUNCH(p, kRowFwd, cs,
                    launch_pdl(k_row_fwd<F>, dim3(a.nb, F / RowCfg<F>::RPB, p.L), row_blk, RowCfg<F>::smem, cs, c.O, c.P, S, a));
-      const dim3 col_grid(F / ColCfg<F>::W, p.G, a.nb);
+      const dim3 col_grid(F / ColCfg<F>::W, a.G, a.nb);
       if (col_staged) {
         rc = narrow ? launch_cols_s<F, 4>(p, true, store, cs, S, Ip, a, aa) : launch_cols_s<F, 0>(p, true, store, cs, S, Ip, a, aa);
         if (rc) return rc;
@@ -373,7 +381,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
     // (with the plain-load columns of the one-field passes also the column adjoint)
     const bool col_plain = !pair && !p.czt && !res && !col_staged && !p.has_tma && p.nchunks == 1;
     auto col_adj_plain = [&](float2* Sp, const KArgs& ap, const AdjArgs& ar) {
-      const dim3 grid(F / ColCfg<F>::W, p.G, ap.nb);
+      const dim3 grid(F / ColCfg<F>::W, a.G, ap.nb);
       auto* kernel = F >= 512 ? (store ? k_col_adj_2b<F, true> : k_col_adj_2b<F, false>)
                               : (store ? k_col_adj<F, true> : k_col_adj<F, false>);
       PTY_LAUNCH(p, kColAdj, cs, launch_pdl(kernel, grid, col_blk, col_adj_smem, cs, Sp, ap, ar));
@@ -407,7 +415,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
     for (int ch = 0; ch < p.nchunks; ++ch) {
       a.chunk_base = ch * p.C;
       a.chunk_len = (LM - a.chunk_base < p.C) ? (LM - a.chunk_base) : p.C;
-      const dim3 col_grid(F / ColCfg<F>::W, p.G, a.nb);
+      const dim3 col_grid(F / ColCfg<F>::W, a.G, a.nb);
       if constexpr (ResSupported<F>::value) {
         if (res) {                                    // Psi recomputed on chip, chi, both gradients
           if (nsets > 1 && k > 0 && cudaStreamWaitEvent(cs, p.ev_radj[(k - 1) % nsets], 0) != cudaSuccess)
@@ -424,7 +432,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
       }
       {
         if (p.czt) {                                  // chirp-z propagator
-          PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_czt_col_adj<F>, dim3(F / CztColCfg<F>::W, p.G, a.nb),
+          PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_czt_col_adj<F>, dim3(F / CztColCfg<F>::W, a.G, a.nb),
                                                 CztColCfg<F>::threads, CztColCfg<F>::smem_adj, cs, S, a, aa, ct));
           if (nsets > 1 && k > 0 && cudaStreamWaitEvent(cs, p.ev_radj[(k - 1) % nsets], 0) != cudaSuccess)
             return PTYCHO_ECUDA;
@@ -440,7 +448,7 @@ int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st) {
         }
       }
       if (pair)
-        PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_col_adj_p<F>, dim3(F / PairCfg<F>::CW, p.G, (a.nb + 1) / 2),
+        PTY_LAUNCH(p, kColAdj, cs, launch_pdl(k_col_adj_p<F>, dim3(F / PairCfg<F>::CW, a.G, (a.nb + 1) / 2),
                                               PairCfg<F>::cthreads, PairCfg<F>::smem_col, cs, p.tmap_pair[set], a, aa));
       if (!store && rerun_rows)
         PTY_LAUNCH(p, kRowFwd, cs,

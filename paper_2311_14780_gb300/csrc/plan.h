@@ -32,7 +32,11 @@ struct ptycho_plan {
 
   // batching: B positions per batch, modes split into chunks of C, columns kernels use
   // G groups of MG modes; store = 1 keeps Psi in S between the forward and the adjoint.
+  // Where one batch takes all positions, a call of at most half of them uses the groups of a third of the
+  // batch (G_few of MG_few modes), which fill the SMs as well with fewer positions.
   int store = 1, B = 1, C = 1, nchunks = 1, G = 1, MG = 1;
+  int G_few = 0, MG_few = 0;                   // 0: G and MG for every call
+  int col_groups = 0;                          // groups asked for by the caller, or 0
   // adjoint row pass over all modes of a wavelength per block (k_row_adj_l): rows per block,
   // position splits (each with its own probe-gradient buffer when nsplit > 1)
   int adj_l = 0, rpb_adj = 1, nsplit_adj = 1;
@@ -44,6 +48,7 @@ struct ptycho_plan {
   // passes over pairs of positions (pair.cuh): the default while all fields of a position fit; rows per
   // block of their row adjoint (its position splits are nsplit_adj)
   int pair = 0, rpb_pair = 1;
+  int nsplit_one = 1;                          // splits of k_row_adj_l in its small calls
   // forward row pass over all modes of a wavelength per block (k_row_fwd_l), same rows per block
   int fwd_l = 0, nsplit_fwd = 1;
   // staged column passes (k_col_fwd_s / k_col_adj_s): one block per W columns of a position
@@ -75,7 +80,8 @@ struct ptycho_plan {
   int32_t* d_rt_idx = nullptr;
   float* d_rt_w = nullptr;
   float2* d_S = nullptr;                       // [nsets][B][C][F][F]
-  float* d_Ipart = nullptr;                    // [nsets][B][G][F][F]
+  float* d_Ipart = nullptr;                    // [nsets][positions][groups][F][F], Ipart_slices frames per set
+  long long Ipart_slices = 0;
   float* d_D = nullptr;                        // [nsets][B][F][F]
   float* d_Gt = nullptr;                       // [nsets][B][F][F] R^T D (remap only)
   double* d_loss_part = nullptr;
@@ -107,7 +113,7 @@ struct ptycho_plan {
   // with a W x min(F, 256) box (column passes); has_tma = 0 falls back to plain loads
   int has_tma = 0;
   alignas(64) CUtensorMap tmap_S[4];
-  // pair passes: each scratch set as [pairs*C*F rows][4 F floats], boxes of one tile's columns
+  // pair passes (the one-field ones above serve their small calls): each scratch set as [pairs*C*F rows][4 F floats], boxes of one tile's columns
   alignas(64) CUtensorMap tmap_pair[4];
   long long bytes = 0;
   long long last_launches = 0;
@@ -182,6 +188,15 @@ constexpr BatchTarget kServeBatchTarget{kServeBatchEvals, 0, 1, 2ll << 30};
 bool reg_args_ok(float mu_l1, float mu_tv, float eta);
 int regularise(ptycho_plan& p, const float2* O, float mu_l1, float mu_tv, float eta, float2* gO, double* loss,
                cudaStream_t st);
+
+// Mode groups (of ``modes`` modes) of the one-field columns in a small call of a plan with pair passes: of nb
+// positions, each with ``colblocks`` blocks per group.
+inline int small_call_groups(const ptycho_plan& p, int colblocks, int nb, int& modes) {
+  const int have = colblocks * nb, want = p.col_groups > 0 ? p.col_groups : (2 * p.sms + have - 1) / have;
+  const int groups = want < p.C ? want : p.C;
+  modes = (p.C + groups - 1) / groups;
+  return (p.C + modes - 1) / modes;
+}
 
 // Defined once per frame size in kern_<F>.cu.
 template <int F> int run_pipeline(ptycho_plan& p, const CallArgs& c, cudaStream_t st);

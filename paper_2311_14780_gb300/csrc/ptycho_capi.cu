@@ -664,20 +664,25 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
     default: colblocks = F / ptycho::ColCfg<512>::W; break;
   }
   const long long want_cols = 2ll * p->sms;   // column blocks wanted: mode groups only below two per SM
-  long long G = (want_cols + (long long)colblocks * p->B - 1) / ((long long)colblocks * p->B);
-  if (p->pair) {                                      // and of the pair passes, in blocks of 128 threads
-    const PairSizes z = pair_sizes(F, g->M, 1);
-    const long long have = (long long)(F / z.CW) * ((p->B + 1) / 2) * z.CW * z.T / 128;
-    G = (want_cols + have - 1) / std::max<long long>(1, have);
-  }
-  if (g->col_groups > 0) G = g->col_groups;
-  G = std::max<long long>(1, std::min<long long>(G, p->C));
-  p->MG = (int)((p->C + G - 1) / G);
-  p->G = (p->C + p->MG - 1) / p->MG;
+  auto mode_groups = [&](int nb, int& groups, int& modes) {   // for launches of nb positions
+    long long have = (long long)colblocks * nb;
+    if (p->pair) {                                    // blocks of the pair passes, in blocks of 128 threads
+      const PairSizes z = pair_sizes(F, g->M, 1);
+      have = std::max<long long>(1, (long long)(F / z.CW) * ((nb + 1) / 2) * z.CW * z.T / 128);
+    }
+    long long G = g->col_groups > 0 ? g->col_groups : (want_cols + have - 1) / have;
+    G = std::max<long long>(1, std::min<long long>(G, p->C));
+    modes = (int)((p->C + G - 1) / G);
+    groups = (p->C + modes - 1) / modes;
+  };
+  mode_groups(p->B, p->G, p->MG);
+  if (p->store && p->B >= g->J && g->J > 1) mode_groups((p->B + 2) / 3, p->G_few, p->MG_few);
+  p->col_groups = std::max(0, g->col_groups);
   if (p->store && (g->flags & PTYCHO_FLAG_STAGED_COLUMNS) && g->col_groups <= 0) {
     p->col_staged = 1;
     p->G = 1;
     p->MG = p->C;
+    p->G_few = 0;
   }
 
   // adjoint row pass over all modes of a wavelength per block (see PTYCHO_FLAG_UNFUSED_ROW_ADJ)
@@ -765,6 +770,7 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
     const long long slots = per_sm * p->sms;
     auto rounds = [&](long long n) { return (n * blocks + slots - 1) / slots; };
     if (g->M > 1 && (ct > 256 || rounds(1) > 1) && 10 * rounds(np) > 9 * rounds(1) * np) np = 1;
+    p->nsplit_one = p->nsplit_adj;                    // of the one-field passes, for small calls
     p->nsplit_adj = (int)std::max<long long>(1, np);
   }
 
@@ -825,7 +831,12 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
   }
   const long long Bs = p->pair ? (p->B + 1) / 2 * 2 : p->B;   // positions of one scratch set (whole pairs)
   rc = rc ? rc : dalloc(p, &p->d_S, (long long)p->nsets * Bs * p->C * FF);
-  rc = rc ? rc : dalloc(p, &p->d_Ipart, (long long)p->nsets * p->B * std::max(p->G, p->res ? p->G_res : 1) * FF);
+  p->Ipart_slices = std::max<long long>((long long)p->B * std::max(p->G, p->res ? p->G_res : 1), (long long)(p->B / 2) * p->G_few);
+  for (int nb = 1; p->pair && nb <= std::min(p->B, ptycho::pair_subset(F)); ++nb) {   // calls through the one-field columns
+    int modes = 0;
+    p->Ipart_slices = std::max<long long>(p->Ipart_slices, (long long)nb * ptycho::small_call_groups(*p, colblocks, nb, modes));
+  }
+  rc = rc ? rc : dalloc(p, &p->d_Ipart, (long long)p->nsets * p->Ipart_slices * FF);
   rc = rc ? rc : dalloc(p, &p->d_D, (long long)p->nsets * p->B * FF);
   rc = rc ? rc : dalloc(p, &p->d_loss_part, (long long)g->J * (FF / (ptycho::kLossThreads * ptycho::kLossPx)));
   rc = rc ? rc : dalloc(p, &p->d_sig_part, (long long)g->J * (FF / (ptycho::kLossThreads * ptycho::kLossPx)));
@@ -835,7 +846,7 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
   rc = rc ? rc : dalloc(p, &p->d_gO, p->O_numel);
   rc = rc ? rc : dalloc(p, &p->d_gP, p->P_numel);
   {
-    const int ns = std::max(p->adj_l_ok || p->pair ? p->nsplit_adj : 1, p->res ? p->nsplit_res : 1);
+    const int ns = std::max(p->adj_l_ok || p->pair ? std::max(p->nsplit_adj, p->nsplit_one) : 1, p->res ? p->nsplit_res : 1);
     if (ns > 1) rc = rc ? rc : dalloc(p, &p->d_gPs, (long long)ns * p->P_numel);
   }
   rc = rc ? rc : dalloc(p, &p->d_status, 1);
@@ -858,9 +869,8 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
     p->has_tma = (g->flags & PTYCHO_FLAG_NO_TMA) || p->czt ? 0 : ((g->flags & PTYCHO_FLAG_TMA) || tma_default) ? 1 : 0;
     // F = 512: the staged column passes with the half-size exchange, two blocks per SM
     p->col_tma2 = F == 512 && !(g->flags & PTYCHO_FLAG_COLS_ONE_BLOCK) ? 1 : 0;
-    if (p->pair) p->has_tma = 0;
     for (int i = 0; i < p->nsets; ++i) {
-      if (p->has_tma && !make_column_map(&p->tmap_S[i], p->d_S + (long long)i * p->B * p->C * FF, F, rows, W))
+      if (p->has_tma && !make_column_map(&p->tmap_S[i], p->d_S + (long long)i * Bs * p->C * FF, F, rows, W))
         p->has_tma = 0;
       if (p->pair && !make_pair_map(&p->tmap_pair[i], p->d_S + (long long)i * Bs * p->C * FF, F, Bs / 2 * p->C * F,
                                     pair_sizes(F, g->M, 1).CW)) {

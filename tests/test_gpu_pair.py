@@ -213,3 +213,17 @@ def test_splits_follow_the_rounds_of_blocks(dev, F, L, M, J, splits):
     assert torch.cuda.get_device_properties(dev).multi_processor_count == 152
     assert plan.query(ROW_ADJ_SPLITS) == splits
     plan.close()
+
+
+@pytest.mark.parametrize("F,L,M,flags", [(64, 2, 3, 0), (128, 1, 4, 0), (256, 2, 3, 0), (512, 1, 2, 0), (512, 1, 12, 0),
+                                         (64, 1, 1, 0), (256, 1, 4, ONE_FIELD)])
+def test_subsets_of_every_size_class(dev, F, L, M, flags):
+    """Calls beside the lines where a plan changes its passes and mode groups: one position, the most that take the
+    one-field passes and one more, half of the batch and one more, all but one."""
+    case = _case(dev, F, L, M, 5, 95 + F + M)
+    plan = case.plan(flags=flags)
+    order = np.random.default_rng(F).permutation(case.w.J)
+    assert case.w.J == 25
+    for n in (1, 2, 10, 11, 12, 13, 16, 17, 24):
+        assert_ok(check_all(case, plan, frames=[int(j) for j in order[:n]]))
+    plan.close()
