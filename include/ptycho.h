@@ -165,7 +165,7 @@ typedef struct {
                                8 GiB; three batches per call where each holds 8 Mi elements,
                                else two or one; of equal size within one position (two with
                                the pair passes).  With zoom 1200 fields per batch, and three
-                               batches per call or, below 4 Mi elements and 8 + 4096 / F
+                               batches per call or, below 4 Mi elements and 4 + 2560 / F
                                positions, one.  On PTYCHO_ENOMEM the target is halved, down
                                to 1200 fields or 64 positions.                           */
   int32_t overlap;          /* position batches in flight on separate streams (1..4), each

@@ -197,9 +197,9 @@ namespace {
 // Chirp-z passes: the per-mode row adjoint takes a batch's positions one after another in few blocks, a chain that
 // overlapping batches hide and that grows with the batch.  So they keep batches of kBatchEvals fields (64^2 x 4 x
 // 2 with 128 / 256 of 768 positions 1937 / 2119 us a step), and calls of under kSmallBatchElems / 2 are merged only
-// below 8 + 4096 / F positions (us a step in one batch / three: 64^2 x 5 fields 26 positions 119 / 131, 51 189 /
-// 187, 102 335 / 310; 128^2 x 8: 16 130 / 172, 48 314 / 302; 256^2 x 1: 16 108 / 117, 32 170 / 171, 48 235 / 227;
-// with more elements 128^2 x 30, 26 positions: 669 / 559).
+// below 4 + 2560 / F positions (us a step in one batch / three: 64^2 x 5 fields 26 positions 119 / 131, 50 182 /
+// 178, 64 228 / 206; 128^2 x 5 20 132 / 136, 32 181 / 176; 128^2 x 8 16 130 / 172, 48 314 / 302; 256^2 x 1 8 74 / 95, 32
+// 170 / 171, 48 235 / 227; with more elements 128^2 x 30, 26 positions: 669 / 559).
 constexpr long long kMaxScratch = 8ll << 30;   // default upper bound of one buffer set
 constexpr long long kBatchElems = 320ll << 20; // field elements per batch the default aims for (1280 of 512^2)
 constexpr long long kSmallBatchElems = 8ll << 20;
@@ -540,7 +540,7 @@ int ptycho_plan_create(const ptycho_geom_t* g, ptycho_plan_t** out) {
 namespace ptycho {
 
 // A plan with the given batching, with the pair passes where they apply if ``pairs``.  kNoPairMap: they would
-// apply, but the driver gave no tensor map for their scratch.
+// apply, but the CUDA driver gave no tensor map for their scratch.
 constexpr int kNoPairMap = 1;
 static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pairs, ptycho_plan_t** out) {
   if (!g || !out) return PTYCHO_EINVAL;
@@ -616,7 +616,7 @@ static int make_plan(const ptycho_geom_t* g, const BatchTarget& target, bool pai
       B = std::min<long long>(B, std::max({(evals + LM - 1) / LM, (kBatchRows + LM * F - 1) / (LM * F),
                                            target.min_positions}));
       const long long whole = !g->zoom ? g->J * elems / kSmallBatchElems
-                              : g->J * elems < kSmallBatchElems / 2 && g->J < 8 + 4096 / F ? 1 : kMinBatches;
+                              : g->J * elems < kSmallBatchElems / 2 && g->J < 4 + 2560 / F ? 1 : kMinBatches;
       const long long nmin = std::max<long long>(1, std::min<long long>(kMinBatches, whole));
       B = std::min<long long>(B, std::max<long long>(1, (g->J + nmin - 1) / nmin));
     }

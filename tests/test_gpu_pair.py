@@ -193,8 +193,8 @@ def test_intensity_sum_rounds_once_per_mode(dev, F, M, flags):
     plan.close()
 
 
-@pytest.mark.parametrize("F,fields,J,batch", [(64, 5, 71, 71), (64, 5, 72, 24), (128, 8, 31, 31), (128, 8, 32, 11), (128, 30, 26, 9),
-                                              (64, 8, 768, 128), (512, 1, 15, 15), (512, 1, 16, 6)])
+@pytest.mark.parametrize("F,fields,J,batch", [(64, 5, 43, 43), (64, 5, 44, 15), (128, 8, 23, 23), (128, 8, 24, 8), (128, 30, 20, 7),
+                                              (64, 8, 768, 128), (512, 1, 8, 8), (512, 1, 9, 3)])
 def test_chirp_z_batches(dev, F, fields, J, batch):
     """Chirp-z batches hold 1200 fields (and at least 64 positions); a call is one batch instead of three only with few
     positions and few elements."""
