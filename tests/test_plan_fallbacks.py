@@ -1,4 +1,4 @@
-"""What plan creation falls back to, read from its source (no GPU): a failure of the driver cannot be had
+"""What plan creation falls back to, read from its source (no GPU): a failure of the CUDA driver cannot be had
 on demand."""
 import os
 import re
